@@ -258,8 +258,8 @@ int ftq_status(ftq_ctx* ctx, int* status_host);
 int ftq_set_green_kernel(ftq_ctx* ctx, int kind);
 
 /* Test hook of the failure detection (no counterpart in the paper): every
- * mbarrier wait of the tensor-core kernels (mixed precision: the chain and
- * the Gauss-Jordan G) polls at
+ * mbarrier wait of the tensor-core kernels (the chain of both precisions, and
+ * the mixed path's Gauss-Jordan G) polls at
  * most `polls` times before it gives up; -1 restores the default of 2^24
  * polls.  A wait that gives up latches FTQ_ETIMEOUT (read by ftq_status), the
  * kernel skips its remaining work, drains its own copies and MMAs with the

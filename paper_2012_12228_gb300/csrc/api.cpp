@@ -45,7 +45,8 @@ void free_all(ftq_ctx* c) {
                     c->tab.vidx, c->tab.pair_ptr, c->tab.pair_a, c->tab.pair_b, c->tab.eps, c->tab.h,
                     c->tab.cq, c->tab.vq, c->tab.vqf, c->tab.ksq, c->tab.g0, c->items, c->tab.pk, c->tab.qcube,
                     c->tab.hf, c->phi32, c->xbuf, c->xsum, c->pc_w, c->pc_cnt, c->pc_parent, c->pc_pairs,
-                    c->sq_walker, c->sq_w, c->sq_out, c->Yf, c->tab.eplus, c->trk, c->trk_out, c->items_lr};
+                    c->sq_walker, c->sq_w, c->sq_out, c->Yf, c->tab.eplus, c->trk, c->trk_out, c->items_lr,
+                    c->oz_dig, c->oz_ev, c->oz_cmax, c->tab.ozidx};
     for (void* p : ptrs)
         if (p) cudaFree(p);
 }
@@ -123,8 +124,12 @@ int ftq_init_ueg(ftq_ctx** out, int N, int M, double rs, double theta, double mu
     const size_t W = c->W, MM = (size_t)M * M;
     cudaError_t e = cudaSuccess;
     auto chk = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
+    // the complex128 tensor-core chain keeps its Horner matrices in Y, zbuf and
+    // work (Y and zbuf[0] change places), with columns padded to oz_kp(M)
+    const bool oz = opts->precision == FTQ_FP64 && !ftq::oz_chain_small(M);
+    const size_t MZ = oz ? (size_t)M * ftq::oz_kp(M) : MM;
     if (opts->precision == FTQ_FP64 || opts->low_rank_threshold > 0.0) {
-        chk(dalloc(c, &c->Y, W * MM));      // the mixed low-rank path keeps a complex128 copy of the chain
+        chk(dalloc(c, &c->Y, W * MZ));      // the mixed low-rank path keeps a complex128 copy of the chain
     }
     if (opts->precision != FTQ_FP64) {
         c->Kp = (M + 15) / 16 * 16;       // 2 Kp is a whole number of 32-float k tiles
@@ -144,10 +149,15 @@ int ftq_init_ueg(ftq_ctx** out, int N, int M, double rs, double theta, double mu
     }
     chk(dalloc(c, &c->Tinv, W * MM));
     chk(dalloc(c, &c->G, W * MM));
-    chk(dalloc(c, &c->work, W * MM));
+    chk(dalloc(c, &c->work, W * MZ));
     chk(dalloc(c, &c->work2, W * MM));
-    chk(dalloc(c, &c->zbuf[0], W * MM));
-    chk(dalloc(c, &c->zbuf[1], W * MM));
+    chk(dalloc(c, &c->zbuf[0], W * MZ));
+    chk(dalloc(c, &c->zbuf[1], W * MZ));
+    if (oz) {
+        chk(dalloc(c, &c->oz_dig, W * c->nslot * 2));
+        chk(dalloc(c, &c->oz_ev, W));
+        chk(dalloc(c, &c->oz_cmax, (size_t)(opts->exp_order + 1) * W * M));
+    }
     chk(dalloc(c, &c->DR, W * M));
     chk(dalloc(c, &c->phi, W * c->nslot));
     if (e == cudaSuccess) chk(cudaMemset(c->phi, 0, sizeof(double2) * W * c->nslot));
@@ -200,6 +210,7 @@ int ftq_init_ueg(ftq_ctx** out, int N, int M, double rs, double theta, double mu
         }
         chk(upload(c, &c->tab.hf, hf));
         chk(upload(c, &c->tab.qcube, s.qcube));
+        if (oz) chk(upload(c, &c->tab.ozidx, ftq::oz_slots(s)));
         // exchange work units: chunks of 32 pairs of every odd (+Q) slot
         std::vector<int4> eplus;
         for (int sl = 1; sl < c->nslot; sl += 2)

@@ -112,23 +112,6 @@ __device__ __forceinline__ void gen_barrier() {
     asm volatile("bar.sync 1, %0;" ::"n"(NGEN) : "memory");
 }
 
-// Bounded wait that also gives up once another warp has latched an abort;
-// the result is uniform over the calling warp's active lanes.
-__device__ bool mbar_wait_ab(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status,
-                             long long limit) {
-    bool ok = false;
-    for (long long i = 0; i < limit && !ok; ++i) {
-        if (*abort_flag) break;
-        ok = mbar_try_wait(bar, parity);
-    }
-    ok = __all_sync(__activemask(), ok);
-    if (!ok && !*abort_flag) {
-        *abort_flag = 1;
-        atomicOr(status, 2);
-    }
-    return ok;
-}
-
 __global__ void __launch_bounds__(NTHREADS_WS, 1) k_chain_tc(const __grid_constant__ TcBatch tb,
                                                              const int4* __restrict__ items, int nitems) {
     extern __shared__ unsigned char smem_raw[];

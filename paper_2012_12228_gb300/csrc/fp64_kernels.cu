@@ -1,8 +1,7 @@
-// Complex128 kernels of the walker slice: force bias and HS fields, the
-// Taylor-Horner application of B to the chain, Householder QRCP
-// stabilisation, and the two-sided stable Green's function with ln det and
-// the phaseless weight (the estimators are in estimators.cu).  One walker per thread block
-// for the factorisations; tiled batched GEMM for the chain.
+// Complex128 kernels of the walker slice: force bias and HS fields, Householder
+// QRCP stabilisation, and the two-sided stable Green's function with ln det and
+// the phaseless weight (the chain is in chain_oz.cu, the estimators in
+// estimators.cu).  One walker per thread block for the factorisations.
 #include <cmath>
 
 #include "block_reduce.cuh"
@@ -89,78 +88,6 @@ __global__ void k_force_bias(const GT* __restrict__ G, const double* __restrict_
         ws[(long)WSTRIDE * w + 5] = gauss.x;
         ws[(long)WSTRIDE * w + 6] = gauss.y;
     }
-}
-
-// ---------------------------------------------------------------- chain GEMM
-// out[i][c] = os_i (us_i Yu[i][c] + alpha sum_k V[i][k] zs_k Zin[k][c]),
-// V[i][k] = phi[vidx[i][k]]: one Horner step of exp(V) applied to the chain.
-constexpr int CT = 32;   // output tile
-constexpr int CK = 16;   // k tile
-
-__global__ void __launch_bounds__(256) k_chain_step(const double2* __restrict__ Zin, const double2* __restrict__ Yu,
-                                                   double2* __restrict__ out, const double2* __restrict__ phi,
-                                                   const uint16_t* __restrict__ vidx, const double* __restrict__ zs,
-                                                   const double* __restrict__ us, const double* __restrict__ os,
-                                                   double alpha, int M, int nslot, int tiles,
-                                                   const double* __restrict__ rank_ws) {
-    __shared__ double2 As[CK][CT + 1];
-    __shared__ double2 Bs[CK][CT + 1];
-    const int w = blockIdx.y;
-    const int ti = blockIdx.x / tiles, tj = blockIdx.x % tiles;
-    const int r0 = ti * CT, c0 = tj * CT;
-    // low rank: only the first m columns of the chain are live
-    if (rank_ws && c0 >= (int)rank_ws[(long)WSTRIDE * w + 12]) return;
-    const long off = (long)w * M * M;
-    const double2* Z = Zin + off;
-    const double2* ph = phi + (long)w * nslot;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    double2 acc[2][2];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 2; ++b) acc[a][b] = make_double2(0.0, 0.0);
-    for (int k0 = 0; k0 < M; k0 += CK) {
-#pragma unroll
-        for (int l = 0; l < 2; ++l) {
-            int e = threadIdx.x + 256 * l;        // 0..511
-            int r = e >> 4, kk = e & 15;          // A tile: 32 rows x 16 k
-            int i = r0 + r, k = k0 + kk;
-            double2 v = make_double2(0.0, 0.0);
-            if (i < M && k < M) v = ph[vidx[(long)i * M + k]];
-            As[kk][r] = v;
-            int kb = e >> 5, cb = e & 31;         // B tile: 16 k x 32 cols
-            int kr = k0 + kb, cc = c0 + cb;
-            double2 z = make_double2(0.0, 0.0);
-            if (kr < M && cc < M) {
-                z = Z[(long)kr * M + cc];
-                if (zs) z = z * zs[kr];
-            }
-            Bs[kb][cb] = z;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < CK; ++kk) {
-            double2 a0 = As[kk][ty], a1 = As[kk][ty + 16];
-            double2 b0 = Bs[kk][tx], b1 = Bs[kk][tx + 16];
-            acc[0][0] = cfma(a0, b0, acc[0][0]);
-            acc[0][1] = cfma(a0, b1, acc[0][1]);
-            acc[1][0] = cfma(a1, b0, acc[1][0]);
-            acc[1][1] = cfma(a1, b1, acc[1][1]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-            int i = r0 + ty + 16 * a, c = c0 + tx + 16 * b;
-            if (i < M && c < M) {
-                long e = off + (long)i * M + c;
-                double2 v = Yu[e] * us[i] + acc[a][b] * alpha;
-                if (os) v = v * os[i];
-                out[e] = v;
-            }
-        }
 }
 
 // ---------------------------------------------------------------- QRCP
@@ -488,28 +415,7 @@ cudaError_t launch_force_bias(ftq_ctx* c, const double* x) {
 }
 
 cudaError_t launch_chain(ftq_ctx* c) {
-    if (c->opts.precision != FTQ_FP64) return mixed_chain(c);
-    const int M = c->M, p = c->opts.exp_order;
-    const int tiles = (M + CT - 1) / CT;
-    dim3 grid(tiles * tiles, c->W);
-    // Horner: Z_p = h Y + V h Y / p;  Z_j = h Y + V Z_{j+1} / j;  Y' = h Z_1
-    const double2* zin = c->Y;
-    int cur = 0;
-    for (int j = p; j >= 1; --j) {
-        double2* out = c->zbuf[cur];
-        LaunchScope ls(c, FTQ_K_CHAIN);
-        k_chain_step<<<grid, 256, 0, c->stream>>>(zin, c->Y, out, c->phi, c->tab.vidx,
-                                                  j == p ? c->tab.h : nullptr, c->tab.h,
-                                                  j == 1 ? c->tab.h : nullptr, 1.0 / j, M, c->nslot, tiles,
-                                                  c->opts.low_rank_threshold > 0.0 ? c->wstate : nullptr);
-        zin = out;
-        cur ^= 1;
-    }
-    // the result sits in zbuf[cur ^ 1]; make it the chain
-    double2* res = c->zbuf[cur ^ 1];
-    c->zbuf[cur ^ 1] = c->Y;
-    c->Y = res;
-    return cudaGetLastError();
+    return c->opts.precision != FTQ_FP64 ? mixed_chain(c) : oz_chain(c);
 }
 
 cudaError_t launch_qrcp64(ftq_ctx* c, const double2* Yin, double2* Qout) {

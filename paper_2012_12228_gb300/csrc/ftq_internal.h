@@ -65,6 +65,7 @@ struct DevTables {
     double* g0 = nullptr;         // diagonal of G(0) = (I + B_T^n)^-1 [M]
     int* pk = nullptr;            // packed basis coordinates [M]
     float2* hf = nullptr;         // h as float pairs (hi, lo) [M]
+    uint16_t* ozidx = nullptr;    // vidx in 64-row blocks with rows of Kp entries, zero padded (complex128 chain)
     uint16_t* qcube = nullptr;    // difference -> slot [S^3]
     int4* eplus = nullptr;        // exchange work units: per half-space transfer (odd slot) and chunk
                                   // of 32 of its pairs, {first, end of the slot's pair list, first pair
@@ -88,6 +89,11 @@ struct ftq_ctx {
     double2* work = nullptr;      // LU / QR workspace                        [W][M][M]
     double2* work2 = nullptr;     // triangular-solve workspace (column-major)[W][M][M]
     double2* zbuf[2] = {nullptr, nullptr};   // Horner buffers (FP64) / FP64 bridges (mixed)
+    // complex128 chain on the tensor cores (chain_oz.cu): the field table as bf16
+    // digits, its exponent per walker, column maxima of every Horner step
+    uint4* oz_dig = nullptr;      //                                           [W][nslot][2]
+    int* oz_ev = nullptr;         //                                           [W]
+    uint32_t* oz_cmax = nullptr;  //                                           [exp_order + 1][W][M]
     // mixed precision: the chain in FP32 planes split hi + lo for 3xTF32,
     // per walker [hi re | hi im | lo re | lo im], each Kp x LD, zero padded
     int Kp = 0, LD = 0;
@@ -245,6 +251,13 @@ cudaError_t green_autotune(ftq_ctx* c, float* ms_tc, float* ms_lu);
 // Pre-pivoted stabilisation of the mixed chain (qr_mixed.cu).
 cudaError_t launch_qr_prepiv(ftq_ctx* c);
 cudaError_t qr_autotune(ftq_ctx* c, int* best_nb, float* best_ms);
+
+// Complex128 chain (chain_oz.cu): one launch for small bases, else tensor-core
+// digit products.
+bool oz_chain_small(int M);
+int oz_kp(int M);
+std::vector<uint16_t> oz_slots(const UegSetup& s);
+cudaError_t oz_chain(ftq_ctx* c);
 
 // Tensor-core chain (chain_tc.cu).
 void tc_plan(int M, int nct, int* R, int* NT);

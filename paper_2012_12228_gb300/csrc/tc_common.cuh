@@ -1,6 +1,7 @@
 // Inline-PTX wrappers for the sm_103a tensor-core kernels: mbarriers, TMA
-// loads, TMEM allocation and loads, tcgen05.mma kind::tf32 with both operands
-// in 128-byte swizzled K-major shared memory, and the descriptors they take.
+// loads, TMEM allocation and loads, tcgen05.mma kind::tf32 and kind::f16 with
+// both operands in 128- or 64-byte swizzled K-major shared memory, and the
+// descriptors they take.
 #pragma once
 #include <cstdint>
 #include <cuda.h>
@@ -83,6 +84,17 @@ __device__ __forceinline__ void mma_tf32(uint32_t dtmem, uint64_t adesc, uint64_
         : "memory");
 }
 
+// The same for kind::f16 operands (both bf16 here).
+__device__ __forceinline__ void mma_f16(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                        uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
+        ::"r"(dtmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                  : "memory");
@@ -101,6 +113,17 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* v) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// 8 consecutive TMEM columns, not waited for: tmem_wait_ld() before use.
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* v) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+        : "r"(taddr)
+        : "memory");
+}
+
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
 // Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups
 // 1024 bytes apart (SBO), descriptor version 1.
 __device__ __forceinline__ uint64_t sdesc_sw128(const void* p) {
@@ -111,6 +134,45 @@ __device__ __forceinline__ uint64_t sdesc_sw128(const void* p) {
     d |= (uint64_t)1 << 46;               // version
     d |= (uint64_t)2 << 61;               // SWIZZLE_128B
     return d;
+}
+
+// The same with 64-byte rows and the 64-byte swizzle (8-row groups 512 bytes apart).
+__device__ __forceinline__ uint64_t sdesc_sw64(const void* p) {
+    uint64_t d = 0;
+    d |= (uint64_t)((smem_u32(p) >> 4) & 0x3FFF);
+    d |= (uint64_t)1 << 16;
+    d |= (uint64_t)(512 >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)4 << 61;               // SWIZZLE_64B
+    return d;
+}
+
+// Instruction descriptor: D f32, A and B bf16, both K-major, M = 128, N = n.
+__device__ __forceinline__ uint32_t idesc_bf16(int n) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+}
+
+// Byte offset of 16-byte chunk q (0..3) of row r in the 64-byte swizzled
+// layout: the chunk index XOR-ed with (r / 2) mod 4.
+__device__ __forceinline__ uint32_t sw64_off(int r, int q) {
+    return (uint32_t)(r * 64 + ((q ^ ((r >> 1) & 3)) << 4));
+}
+
+// Bounded wait that also gives up once another warp has latched an abort;
+// the result is uniform over the calling warp's active lanes.
+__device__ __forceinline__ bool mbar_wait_ab(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status,
+                                             long long limit) {
+    bool ok = false;
+    for (long long i = 0; i < limit && !ok; ++i) {
+        if (*abort_flag) break;
+        ok = mbar_try_wait(bar, parity);
+    }
+    ok = __all_sync(__activemask(), ok);
+    if (!ok && !*abort_flag) {
+        *abort_flag = 1;
+        atomicOr(status, 2);
+    }
+    return ok;
 }
 
 // Instruction descriptor: D f32, A and B tf32, both K-major, M = 128, N = n
