@@ -206,7 +206,8 @@ def kernel_model(kind, M, W, precision, green_tc=False):
             return (3 * 8.0 * M ** 3 * W,) + tf32
         return (8.0 * M ** 3 * W,) + (fp64 if precision == "fp64" else fp32)
     if kind == "green":
-        if green_tc:             # Gauss-Jordan on [Mt^T | B^T]: 1.5 M^3 complex MACs, as 3xTF32 MMAs
+        if green_tc:             # elimination of [Mt^T | B^T] on the tensor cores, counted as 1.5 M^3 complex
+                                 # MACs at tf32 cost (six bf16 products each; the blocked LU needs 4/3 M^3)
             return (3 * 12.0 * M ** 3 * W,) + tf32
         # LU (8/3 M^3) + two triangular solves with M right-hand sides (8 M^3)
         return ((8.0 / 3.0 + 8.0) * M ** 3 * W,) + (fp64 if precision == "fp64" else fp32)
@@ -261,7 +262,7 @@ def measure_path(ftq, torch, dev, precision, W, steps, warmup, world, rank, barr
     out = {"M": M, "n_slices": n, "dtau": prop.query_f64("DTAU"), "walkers": W, "stab": stab, "p": p_order,
            "autotune": None if tuned is None else {"column_tiles": tuned[0], "ms_per_horner_step": tuned[1],
                                                    "qr_panel": prop.query("QR_PANEL"),
-                                                   "green_kernel": {1: "tensor-core Gauss-Jordan",
+                                                   "green_kernel": {1: "blocked LU, tensor-core updates",
                                                                     2: "CUDA-core blocked LU"}.get(
                                                        prop.query("GREEN_KERNEL"), "none")}}
 

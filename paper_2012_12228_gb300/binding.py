@@ -350,7 +350,7 @@ class Propagator:
                 "N_avg": complex(a[0, 3], a[0, 4])}
 
     def set_green_kernel(self, kind):
-        """Mixed path's G(tau) kernel: 0 by basis size, 1 tensor cores (Gauss-Jordan), 2 CUDA cores (LU)."""
+        """Mixed path's G(tau) kernel: 0 by basis size, 1 tensor-core updates, 2 CUDA cores (both LU)."""
         self._check(self.lib.ftq_set_green_kernel(self.h, int(kind)), "ftq_set_green_kernel")
 
     def set_wait_limit(self, polls):

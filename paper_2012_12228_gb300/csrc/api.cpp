@@ -1,5 +1,6 @@
 // C ABI of the walker-propagation library: context lifetime, device
 // allocations, and the per-slice launch sequence.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -39,14 +40,14 @@ cudaError_t upload(ftq_ctx* c, T** p, const std::vector<T>& v) {
 }
 
 void free_all(ftq_ctx* c) {
-    void* ptrs[] = {c->Y, c->Tinv, c->G, c->work, c->work2, c->zbuf[0], c->zbuf[1], c->DR, c->phi,
+    void* ptrs[] = {c->Y, c->Tinv, c->G, c->work, c->zbuf[0], c->zbuf[1], c->DR, c->phi,
                     c->Ypl, c->zpl[0], c->zpl[1], c->G32, c->w32,
                     c->hh, c->htau, c->perm, c->wstate, c->est, c->red, c->status,
                     c->tab.vidx, c->tab.pair_ptr, c->tab.pair_a, c->tab.pair_b, c->tab.eps, c->tab.h,
                     c->tab.cq, c->tab.vq, c->tab.vqf, c->tab.ksq, c->tab.g0, c->items, c->tab.pk, c->tab.qcube,
                     c->tab.hf, c->phi32, c->xbuf, c->xsum, c->pc_w, c->pc_cnt, c->pc_parent, c->pc_pairs,
                     c->sq_walker, c->sq_w, c->sq_out, c->Yf, c->tab.eplus, c->trk, c->trk_out, c->items_lr,
-                    c->oz_dig, c->oz_ev, c->oz_cmax, c->tab.ozidx};
+                    c->oz_dig, c->oz_ev, c->oz_cmax, c->tab.ozidx, c->lu_scal, c->lu_int};
     for (void* p : ptrs)
         if (p) cudaFree(p);
 }
@@ -140,17 +141,18 @@ int ftq_init_ueg(ftq_ctx** out, int N, int M, double rs, double theta, double mu
         chk(dalloc(c, &c->zpl[0], W * wsz));
         chk(dalloc(c, &c->zpl[1], W * wsz));
         chk(dalloc(c, &c->G32, W * MM));
-        // one allocation: the LU and solve halves for the QR and blocked LU
-        // kernels, or per walker one contiguous M x 2M complex block for the
-        // tensor-core Gauss-Jordan Green kernel
-        chk(dalloc(c, &c->w32, W * std::max(2 * MM, (ftq::green_tc_floats(M) + 1) / 2)));
+        // one allocation: the LU and solve halves for the QR and CUDA-core LU
+        // kernels, or per walker one M x lu_ld(M) block for the tensor-core LU
+        chk(dalloc(c, &c->w32, W * M * ftq::lu_ld(M)));
         c->w2_32 = c->w32 + W * MM;
         chk(dalloc(c, &c->xsum, W * MM));
     }
     chk(dalloc(c, &c->Tinv, W * MM));
     chk(dalloc(c, &c->G, W * MM));
-    chk(dalloc(c, &c->work, W * MZ));
-    chk(dalloc(c, &c->work2, W * MM));
+    chk(dalloc(c, &c->work, W * std::max(MZ, (size_t)M * ftq::lu_ld(M))));
+    c->work2 = c->work + W * MM;
+    chk(dalloc(c, &c->lu_scal, ftq::lu_scal_doubles(M, (int)W)));
+    chk(dalloc(c, &c->lu_int, ftq::lu_ints((int)W)));
     chk(dalloc(c, &c->zbuf[0], W * MZ));
     chk(dalloc(c, &c->zbuf[1], W * MZ));
     if (oz) {
@@ -227,6 +229,7 @@ int ftq_init_ueg(ftq_ctx** out, int N, int M, double rs, double theta, double mu
         }
         chk(ftq::tc_make_maps(c));
     }
+    if (e == cudaSuccess) chk(ftq::lu_make_maps(c));
     if (e == cudaSuccess) chk(cudaMemsetAsync(c->status, 0, sizeof(int), c->stream));
     if (e == cudaSuccess) chk(ftq::launch_init_walkers(c));
     if (e != cudaSuccess) {

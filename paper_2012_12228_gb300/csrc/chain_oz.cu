@@ -44,6 +44,7 @@
 #include <vector>
 
 #include "complex_math.cuh"
+#include "digits.cuh"
 #include "ftq_internal.h"
 #include "tc_common.cuh"
 
@@ -62,9 +63,6 @@ constexpr int NSTAGE = 2;
 constexpr int W_EPI = 4, W_A = 8, W_B = 4;
 constexpr int NT_OZ = 32 * (W_EPI + W_A + W_B + 1);
 constexpr int CHUNK_K = 256;                // complex k whose products one accumulator sums
-// bias that makes the digits of a signed integer non-negative: 64 (1 + 128 + .. + 128^6)
-constexpr long long DBIAS = 64LL * (((1LL << 49) - 1) / 127);
-
 // Planes of a complex128 chain matrix: column c of walker w at
 // ((w M + c) 2 + part) Kp, rows contiguous.
 struct OzArgs {
@@ -90,40 +88,6 @@ __device__ __forceinline__ int item_of(int t, int per, int n, bool spread) {
     // ranks, spread over the CTAs so that skipped tiles leave them balanced
     const int it = spread ? t * (int)gridDim.x + (int)blockIdx.x : (int)blockIdx.x * per + t;
     return it < n && (spread || t < per) ? it : -1;
-}
-
-// 64-bit integer round(|v| 2^s) with the sign of v, for a column (or table)
-// whose largest exponent field is E: s puts E's values below 2^(53 + up).
-__device__ __forceinline__ long long fixed_point(double v, int E, int up) {
-    const long long b = __double_as_longlong(v);
-    const int e = (int)((b >> 52) & 0x7ff);
-    const unsigned long long m = e > 0 ? (((unsigned long long)b & 0xfffffffffffffULL) | (1ULL << 52)) : 0ULL;
-    int rs = E - e;
-    rs = rs < 0 ? 0 : (rs > 62 ? 62 : rs);
-    const unsigned long long half = rs > 0 ? (1ULL << (rs - 1)) : 0ULL;
-    const long long f = (long long)(((m << up) + half) >> rs);
-    return b < 0 ? -f : f;
-}
-
-// bf16 bits (upper half of the FP32 word) of the eight digits of f.
-__device__ __forceinline__ void digits8(long long f, float (&d)[ND]) {
-    const long long g = f + DBIAS;
-    const uint32_t lo = (uint32_t)g;
-    const int hi = (int)(g >> 32);
-    const uint32_t mid = __funnelshift_r(lo, (uint32_t)hi, 28);
-    d[0] = (float)(hi >> 17);
-    const uint32_t u[7] = {(uint32_t)hi >> 10, (uint32_t)hi >> 3, mid, lo >> 21, lo >> 14, lo >> 7, lo};
-#pragma unroll
-    for (int j = 0; j < 7; ++j) d[j + 1] = __uint_as_float((u[j] & 127u) | 0x4B000000u) - 8388672.0f;
-}
-
-__device__ __forceinline__ uint32_t pack_hi(float a, float b) {
-    return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
-}
-
-// v 2^n, in one multiplication where 2^n is a normal number.
-__device__ __forceinline__ double scale_pow2(double v, int n) {
-    return n > -1000 && n < 1000 ? v * __hiloint2double((1023 + n) << 20, 0) : scalbn(v, n);
 }
 
 __device__ __forceinline__ void a_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(32 * W_A) : "memory"); }
@@ -197,7 +161,9 @@ __global__ void __launch_bounds__(NT_OZ, 1) k_chain_oz(const OzArgs p) {
         }
     } else if (warp >= W_EPI + W_A) {
         // ------------------------------------------------ digits of Z
-        const int c = lane, kq = warp - (W_EPI + W_A);     // column, group of 4 complex k
+        // column, group of 4 complex k (lanes 8..15 and 24..31 take the neighbour's, so that the 8-byte
+        // stores of a half warp meet no bank twice)
+        const int c = lane, kq = (warp - (W_EPI + W_A)) ^ ((lane >> 3) & 1);
         const uint32_t o_re = sw64_off(c, kq >> 1) + (uint32_t)(kq & 1) * 8u;
         const uint32_t o_im = sw64_off(c, 2 + (kq >> 1)) + (uint32_t)(kq & 1) * 8u;
         int g = 0;
@@ -341,14 +307,10 @@ __global__ void __launch_bounds__(NT_OZ, 1) k_chain_oz(const OzArgs p) {
                     for (int q = 0; q < 8; ++q) {
                         const int c = col0 + cc + q;
                         if (c >= p.M) break;         // uniform over the warp
-                        auto lev = [&](int l) { return (long long)__float2int_rn(__uint_as_float(v[l][q])); };
-                        const long long h = (lev(0) << 21) + (lev(1) << 14) + (lev(2) << 7) + lev(3);
-                        const long long m = (lev(4) << 21) + (lev(5) << 14) + (lev(6) << 7) + lev(7);
-                        // |h|, |m| < 2^47: exact in FP64, by adding 1.5 2^52 in the integer domain
-                        const double magic = 6755399441055744.0;
-                        const double hd = __longlong_as_double(__double_as_longlong(magic) + h) - magic;
-                        const double md = __longlong_as_double(__double_as_longlong(magic) + m) - magic;
-                        const double sum = fma(hd, 268435456.0, md);       // levels 0..3 weigh 2^28 more
+                        float lv[ND];
+#pragma unroll
+                        for (int l = 0; l < ND; ++l) lv[l] = __uint_as_float(v[l][q]);
+                        const double sum = level_sum(lv);
                         // V is scaled by 2^(1078 - ev), Z by 2^(1079 - ec); the level-7 unit of the
                         // product weighs 2^49 (digit weights 2^(49 - 7 j) of both factors)
                         const int ec = (int)(p.cin[(size_t)w * p.M + c] >> 20);

@@ -476,6 +476,18 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 
 }  // namespace
 
+// Tensor map of a [nz][ny][nx] FP32 array (strides in bytes) in boxes of
+// by rows of bx floats, unswizzled.
+bool tc_map_3d(void* map, void* base, size_t nx, size_t ny, size_t nz, size_t sy, size_t sz, int bx, int by) {
+    PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
+    if (!enc) return false;
+    cuuint64_t dims[3] = {nx, ny, nz}, strides[2] = {sy, sz};
+    cuuint32_t box[3] = {(cuuint32_t)bx, (cuuint32_t)by, 1}, estr[3] = {1, 1, 1};
+    return enc(reinterpret_cast<CUtensorMap*>(map), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // Tile plan for basis size M with nct column tiles: rows covered by 64-row
 // MMA blocks (R, possibly padded above M) and the MMA N width (<= 256).
 void tc_plan(int M, int nct, int* R, int* NT) {

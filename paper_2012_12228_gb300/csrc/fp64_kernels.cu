@@ -7,11 +7,10 @@
 #include "block_reduce.cuh"
 #include "complex_math.cuh"
 #include "ftq_internal.h"
+#include "green_tail.cuh"
 
 namespace ftq {
 namespace {
-
-constexpr double kPi = 3.14159265358979323846;
 
 // ---------------------------------------------------------------- init
 __global__ void k_init_matrices(double2* Y, double2* Tinv, double2* G, const double* g0, int M, long total) {
@@ -334,40 +333,8 @@ __global__ void k_green(const double2* __restrict__ Y, const double2* __restrict
     for (int i = threadIdx.x; i < M; i += nt) trg = trg + Gw[(long)i * M + i];
     trg = block_sum(trg, shc);
     if (threadIdx.x == 0) {
-        double* s = ws + (long)WSTRIDE * w;
-        double2 ld = ldm;
-        ld.x -= lsum;
-        ld.y += kPi * (double)(nswap ^ ((int)s[7]));
-        if (!isfinite(ld.x) || !isfinite(ld.y)) atomicOr(status, 1);
-        // d ln det(I + A_k)/dmu = k dtau (M - tr G(tau_k)): every B carries exp(dtau mu)
-        const double2 tk = make_double2(kdt * ((double)M - trg.x), -kdt * trg.y);
-        if (update) {
-            double2 lnS = make_double2(2.0 * (ld.x - s[3]), 2.0 * (ld.y - s[4]));
-            const double2 dlnS = make_double2(2.0 * (tk.x - s[9]), 2.0 * (tk.y - s[10]));
-            const double gr = with_gauss ? s[5] : 0.0, gi = with_gauss ? s[6] : 0.0;
-            if (constraint == FTQ_FREE) {
-                s[0] += lnS.x + gr;
-                s[1] = remainder(s[1] + lnS.y + gi, 2.0 * kPi);
-                s[8] += dlnS.x;
-                s[11] += dlnS.y;
-            } else if (s[2] > 0.5) {
-                const double cth = cos(lnS.y);
-                if (!isfinite(lnS.x + gr) || !(cth == cth)) {
-                    // a non-finite ratio or Gaussian factor drops the walker (weight 0)
-                    s[2] = 0.0;
-                    atomicOr(status, 1);
-                } else if (cth <= 0.0) {
-                    s[2] = 0.0;
-                } else {
-                    s[0] += lnS.x + gr + log(cth);
-                    s[8] += dlnS.x - tan(lnS.y) * dlnS.y;   // d log cos(theta) = -tan(theta) d theta
-                }
-            }
-        }
-        s[3] = ld.x;
-        s[4] = remainder(ld.y, 2.0 * kPi);
-        s[9] = tk.x;
-        s[10] = tk.y;
+        green_weight_tail(ws + (long)WSTRIDE * w, ldm, lsum, nswap, trg, M, kdt, constraint, status, update,
+                          with_gauss);
     }
 }
 
@@ -445,9 +412,10 @@ double left_scale(const ftq_ctx* c, int k) {
 
 cudaError_t launch_green64(ftq_ctx* c, const double2* Y, int k, bool update, bool physical) {
     const int M = c->M;
+    if (c->opts.low_rank_threshold > 0.0) return launch_green_lr(c, Y, k, update, physical);
+    if (lu64_supported(M)) return launch_green_lu64(c, Y, k, update, physical);
     size_t sm = (2 * sizeof(double2) + 3 * sizeof(double) + sizeof(int)) * M;
     int nt = fact_threads(M);
-    if (c->opts.low_rank_threshold > 0.0) return launch_green_lr(c, Y, k, update, physical);
     const double lscale = physical ? 0.0 : left_scale(c, k);
     if (sm > 48 * 1024) cudaFuncSetAttribute(k_green, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     LaunchScope ls(c, FTQ_K_GREEN);

@@ -86,14 +86,17 @@ struct ftq_ctx {
     double2* Y = nullptr;         // FP64 chain: B's since the last QRCP times Q_R [W][M][M]
     double2* Tinv = nullptr;      // T_R^-1                                   [W][M][M]
     double2* G = nullptr;         // G(tau_k), complex128                     [W][M][M]
-    double2* work = nullptr;      // LU / QR workspace                        [W][M][M]
-    double2* work2 = nullptr;     // triangular-solve workspace (column-major)[W][M][M]
+    double2* work = nullptr;      // LU / QR workspace, S of the blocked LU   [W][M][lu_ld(M)]
+    double2* work2 = nullptr;     // second half of it (work + W M M): triangular solves
     double2* zbuf[2] = {nullptr, nullptr};   // Horner buffers (FP64) / FP64 bridges (mixed)
     // complex128 chain on the tensor cores (chain_oz.cu): the field table as bf16
     // digits, its exponent per walker, column maxima of every Horner step
     uint4* oz_dig = nullptr;      //                                           [W][nslot][2]
     int* oz_ev = nullptr;         //                                           [W]
     uint32_t* oz_cmax = nullptr;  //                                           [exp_order + 1][W][M]
+    double* lu_scal = nullptr;    // blocked LU Green's function: scales, reciprocal pivots
+    int* lu_int = nullptr;        // its pivot parities and panel permutations
+    alignas(64) unsigned char lu_map[2][128] = {};   // its tensor maps of S: complex64 (w32), complex128 (work)
     // mixed precision: the chain in FP32 planes split hi + lo for 3xTF32,
     // per walker [hi re | hi im | lo re | lo im], each Kp x LD, zero padded
     int Kp = 0, LD = 0;
@@ -241,16 +244,35 @@ cudaError_t launch_mu_grad(ftq_ctx* c, double* per_walker);
 // memory fits.
 size_t green32b_smem(int M);
 cudaError_t launch_green32b(ftq_ctx* c, int k, float2* G = nullptr, double* ws = nullptr);
-size_t green_tc_smem(int M, int NT);
-size_t green_tc_floats(int M);   // workspace floats per walker of the tensor-core Green kernel
-int green_tc_tile(int M);
-cudaError_t launch_green_tc(ftq_ctx* c, int k, float2* G = nullptr, double* ws = nullptr);
 bool green_uses_tc(const ftq_ctx* c);
 cudaError_t green_autotune(ftq_ctx* c, float* ms_tc, float* ms_lu);
 
 // Pre-pivoted stabilisation of the mixed chain (qr_mixed.cu).
 cudaError_t launch_qr_prepiv(ftq_ctx* c);
 cudaError_t qr_autotune(ftq_ctx* c, int* best_nb, float* best_ms);
+
+// Blocked LU Green's function with tensor-core updates (green_lu.cu): its
+// per-walker scales and bookkeeping, and the row length of S = [Mt^T | B^T].
+constexpr int LU_NB_MAX = 32;
+template <typename T> struct LuVec;
+template <> struct LuVec<float> { using type = float2; };
+template <> struct LuVec<double> { using type = double2; };
+template <typename T>
+struct LuScales {
+    T *dlb, *dls, *drb;               // [W][M] trial factors at most one, and the right ones split off
+    typename LuVec<T>::type *drs;     // [W][M]
+    typename LuVec<T>::type *inv;     // [W][M] reciprocal pivots
+    double* lsum;                     // [W] logs of the factors split off
+    int* swaps;                       // [W] pivot parity
+    int* perm;                        // [W][2][LU_NB_MAX] the panel's permutation
+};
+int lu_ld(int M);
+size_t lu_scal_doubles(int M, int W);
+size_t lu_ints(int W);
+bool lu64_supported(int M);
+cudaError_t lu_make_maps(ftq_ctx* c);
+cudaError_t launch_green_lu64(ftq_ctx* c, const double2* Y, int k, bool update, bool physical);
+cudaError_t launch_green_lu32(ftq_ctx* c, int k, float2* G = nullptr, double* ws = nullptr);
 
 // Complex128 chain (chain_oz.cu): one launch for small bases, else tensor-core
 // digit products.
@@ -260,6 +282,7 @@ std::vector<uint16_t> oz_slots(const UegSetup& s);
 cudaError_t oz_chain(ftq_ctx* c);
 
 // Tensor-core chain (chain_tc.cu).
+bool tc_map_3d(void* map, void* base, size_t nx, size_t ny, size_t nz, size_t sy, size_t sz, int bx, int by);
 void tc_plan(int M, int nct, int* R, int* NT);
 cudaError_t tc_chain_step_batch(ftq_ctx* b, const float* const* zin, float* const* out, int j, int p);
 cudaError_t tc_batch_items(ftq_ctx* b);

@@ -469,8 +469,8 @@ cudaError_t mixed_green(ftq_ctx* c, int k) {
         return e;
     }
     if (green_uses_tc(c)) {
-        // rank-16 Gauss-Jordan updates on the tensor cores
-        cudaError_t e = launch_green_tc(c, k);
+        // blocked LU with its updates on the tensor cores
+        cudaError_t e = launch_green_lu32(c, k);
         c->g64_valid = false;
         return e;
     }
@@ -491,17 +491,19 @@ cudaError_t mixed_green(ftq_ctx* c, int k) {
     return cudaGetLastError();
 }
 
-// Which Green kernel the mixed path runs for slices k < n.  The tensor-core
-// Gauss-Jordan kernel streams S = [Mt^T | B^T] once per 16-column panel, the
-// CUDA-core blocked LU computes in shared-memory panels with four walkers per
-// SM; measured per 5-slice block on a GB300: M = 257, 1024 walkers: 96.7 ms
-// (tensor cores) vs 63.6 ms (LU); M = 515, 152 walkers: 86.5 vs 149.1 ms.
-// Without a measurement the crossover is taken between the two basis sizes;
-// ftq_autotune times both on the context's own workload.
-constexpr int GREEN_TC_MIN_M = 384;
+// Which Green kernel the mixed path runs for slices k < n: the blocked LU whose
+// updates run on the tensor cores (green_lu.cu), or the CUDA-core LU with one block
+// per walker.  Measured on a GB300, ms per slice (tensor cores / CUDA cores):
+// M = 7, 64 walkers 0.059 / 0.035; M = 33, 300 walkers 0.130 / 0.114; M = 57, 640
+// walkers 0.240 / 0.437; M = 123, 256 walkers 0.43 / 0.71; M = 257, 1024 walkers
+// 7.5 / 9.4; M = 257, 64 walkers 0.88 / 2.5; M = 515, 64 walkers 3.4 / 17.0.  Without a
+// measurement the tensor cores take over above M = 57, where FP32 rounding of either
+// kernel leaves the drift of the mixed chain least room; ftq_autotune times both on
+// the context's own workload.
+constexpr int GREEN_TC_MIN_M = 64;
 
 bool green_uses_tc(const ftq_ctx* c) {
-    if (c->opts.precision == FTQ_MIXED_SIMT || green_tc_tile(c->M) == 0) return false;
+    if (c->opts.precision == FTQ_MIXED_SIMT) return false;
     if (c->green_kind == 1) return true;
     if (c->green_kind == 2) return false;
     return c->M >= GREEN_TC_MIN_M;
@@ -512,8 +514,7 @@ bool green_uses_tc(const ftq_ctx* c) {
 // (zbuf[0] and est), so that neither G(tau) nor the walker state changes.
 cudaError_t green_autotune(ftq_ctx* c, float* ms_tc, float* ms_lu) {
     *ms_tc = *ms_lu = 0.f;
-    if (c->opts.precision == FTQ_MIXED_SIMT || c->opts.low_rank_threshold > 0.0 || green_tc_tile(c->M) == 0)
-        return cudaSuccess;
+    if (c->opts.precision == FTQ_MIXED_SIMT || c->opts.low_rank_threshold > 0.0) return cudaSuccess;
     float2* gs = reinterpret_cast<float2*>(c->zbuf[0]);
     double* ws = c->est;
     const size_t wbytes = sizeof(double) * WSTRIDE * (size_t)c->W;
@@ -525,7 +526,7 @@ cudaError_t green_autotune(ftq_ctx* c, float* ms_tc, float* ms_lu) {
     cudaEventCreate(&e1);
     const int k = c->k < c->sys.n_slices ? c->k + 1 : 1;
     for (int kind = 1; kind <= 2 && e == cudaSuccess; ++kind) {
-        auto run = [&]() { return kind == 1 ? launch_green_tc(c, k, gs, ws) : launch_green32b(c, k, gs, ws); };
+        auto run = [&]() { return kind == 1 ? launch_green_lu32(c, k, gs, ws) : launch_green32b(c, k, gs, ws); };
         e = cudaMemcpyAsync(ws, c->wstate, wbytes, cudaMemcpyDeviceToDevice, c->stream);
         if (e == cudaSuccess) e = run();                          // warm-up
         if (e == cudaSuccess) e = cudaMemcpyAsync(ws, c->wstate, wbytes, cudaMemcpyDeviceToDevice, c->stream);
@@ -542,7 +543,8 @@ cudaError_t green_autotune(ftq_ctx* c, float* ms_tc, float* ms_lu) {
     // the trial inputs are whatever the chain holds; a flag they raise is not the caller's
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->status, &saved_status, sizeof(int), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    if (e == cudaSuccess) c->green_kind = *ms_tc < *ms_lu ? 1 : 2;
+    // one timed launch each: a tie goes to the single kernel, which needs fewer launches
+    if (e == cudaSuccess) c->green_kind = *ms_tc < 0.95f * *ms_lu ? 1 : 2;
     return e;
 }
 
