@@ -368,23 +368,6 @@ __global__ void __launch_bounds__(NTHREADS_WS, 1) k_chain_tc(const __grid_consta
     if (warp == 0) tmem_dealloc(tmem, 2u * (uint32_t)tb.ncols);
 }
 
-// Output entries outside the MMA tile: rows [R, M) x all columns and
-// columns [NT, M) x rows [0, R), on CUDA cores in FP32 from the same
-// hi + lo operands.  A border row of V (or a border column of Z) is staged in
-// shared memory once and reused for every output of that row (column).
-__device__ __forceinline__ void border_store(float* O, const float* U, const Planes& P, const double* us,
-                                             const double* os, float alpha, int i, int c, float2 acc) {
-    float2 u = P.load(U, i, c);
-    const ScaleF s(us[i]);
-    float2 val = make_float2(fmaf(alpha, acc.x, s(u.x)), fmaf(alpha, acc.y, s(u.y)));
-    if (os) {
-        const ScaleF o(os[i]);
-        val.x = o(val.x);
-        val.y = o(val.y);
-    }
-    P.store(O, i, c, val);
-}
-
 __device__ __forceinline__ float2 warp_sum(float2 v) {
     for (int o = 16; o > 0; o >>= 1) {
         v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
@@ -393,71 +376,131 @@ __device__ __forceinline__ float2 warp_sum(float2 v) {
     return v;
 }
 
-// One warp per output entry, lanes over the contraction index (coalesced
-// reads of the chain rows), V from the shared difference cube.  Eight blocks
-// per SM (at most 32 registers) keep 1024 walkers in one wave, and two
-// partial sums per lane keep eight chain loads in flight.
-__global__ void __launch_bounds__(256, 8) k_chain_border(const float* __restrict__ Zin, const float* __restrict__ Yu,
-                                                     float* __restrict__ out, const double2* __restrict__ phi,
-                                                     const int* __restrict__ pk, const uint16_t* __restrict__ qcube,
-                                                     const double* __restrict__ zs, const double* __restrict__ us,
-                                                     const double* __restrict__ os, float alpha, int M, int nslot,
-                                                     int qsize, int qoff, Planes P, size_t wstride, int R, int NT) {
-    extern __shared__ unsigned char smem_raw[];
-    float2* vec = reinterpret_cast<float2*>(smem_raw);     // [M]: one row of V zs or one column of Z zs
-    float2* phs = vec + M;                                  // [nslot]
-    int* pks = reinterpret_cast<int*>(phs + nslot);         // [M]
-    uint16_t* qs = reinterpret_cast<uint16_t*>(pks + M);    // [qsize]
-    const int w = blockIdx.x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const float* Z = Zin + wstride * w;
-    const float* U = Yu + wstride * w;
-    float* O = out + wstride * w;
-    const double2* ph = phi + (long)w * nslot;
-    const int Rr = R < M ? R : M;
-    for (int e = threadIdx.x; e < nslot; e += blockDim.x) {
-        const double2 d = ph[e];
-        phs[e] = make_float2((float)d.x, (float)d.y);
+// Output entries outside the MMA tile: rows [R, M) x all columns and columns
+// [NT, M) x rows [0, R), on CUDA cores in FP32 from the same hi + lo operands.
+//
+// Border rows: one block per walker and BC columns, a warp per column, lanes over
+// the contraction index (coalesced reads of the chain rows), the NR border rows of
+// V zs staged in shared memory and all of them formed from one pass over Z.
+// What bounds it is reading Z (both planes, 1.1 MB per walker at M = 257) once per
+// Horner step, so the work is spread over columns until the loads of every SM are
+// in flight: at M = 257, 1024 walkers 0.47 -> 0.37 ms per step against one block per
+// walker with the field table and difference cube staged in each, at M = 515 (three
+// border rows), 64 walkers 1.78 -> 0.09 ms.
+constexpr int BC = 32;                  // columns of a block
+constexpr int BORDER_ROWS = 8;          // most border rows of a tile plan
+
+struct BorderArgs {
+    const float* Zin;
+    const float* Yu;
+    float* out;
+    const float2* phi;
+    const uint16_t* vidx;
+    const float2* h;                    // kinetic half step as float pairs
+    float alpha;
+    int M, nslot, R, NT, first, last;   // first / last Horner step: h scales Z / the result
+    Planes P;
+    size_t wstride;
+};
+
+__device__ __forceinline__ void border_store(const BorderArgs& b, int w, int i, int c, float2 acc, float2 u) {
+    const ScaleF s(b.h[i]);
+    float2 val = make_float2(fmaf(b.alpha, acc.x, s(u.x)), fmaf(b.alpha, acc.y, s(u.y)));
+    if (b.last) {
+        val.x = s(val.x);
+        val.y = s(val.y);
     }
-    for (int e = threadIdx.x; e < M; e += blockDim.x) pks[e] = pk[e];
-    for (int e = threadIdx.x; e < qsize; e += blockDim.x) qs[e] = qcube[e];
+    b.P.store(b.out + b.wstride * w, i, c, val);
+}
+
+template <int NR>
+__device__ __forceinline__ void border_rows(const BorderArgs& b, float2* vec, int w, int c0) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, M = b.M;
+    const float* Z = b.Zin + b.wstride * w;
+    const float2* ph = b.phi + (size_t)w * b.nslot;
+    for (int e = threadIdx.x; e < NR * M; e += blockDim.x) {
+        const int i = b.R + e / M, k = e % M;
+        const ScaleF sk(b.first ? b.h[k] : make_float2(1.f, 0.f));
+        const float2 v = ph[b.vidx[(size_t)i * M + k]];
+        vec[e] = make_float2(sk(v.x), sk(v.y));
+    }
     __syncthreads();
-    for (int i = Rr; i < M; ++i) {              // border rows: (V zs)[i, :] Z
-        for (int k = threadIdx.x; k < M; k += blockDim.x) {
-            const ScaleF sk(zs ? zs[k] : 1.0);
-            const float2 v = phs[qs[pks[i] - pks[k] + qoff]];
-            vec[k] = make_float2(sk(v.x), sk(v.y));
-        }
-        __syncthreads();
-        for (int c = warp; c < M; c += nw) {
-            float2 acc = make_float2(0.f, 0.f), acc2 = make_float2(0.f, 0.f);
-            int k = lane;
-            for (; k + 32 < M; k += 64) {
-                const float2 z0 = P.load(Z, k, c), z1 = P.load(Z, k + 32, c);
-                acc = cfma(vec[k], z0, acc);
-                acc2 = cfma(vec[k + 32], z1, acc2);
+    for (int c = c0 + warp; c < min(M, c0 + BC); c += 8) {
+        float2 acc[NR], acc2[NR];
+#pragma unroll
+        for (int r = 0; r < NR; ++r) acc[r] = acc2[r] = make_float2(0.f, 0.f);
+        float2 u[NR];                                      // the U term, on its way during the sum
+#pragma unroll
+        for (int r = 0; r < NR; ++r) u[r] = b.P.load(b.Yu + b.wstride * w, b.R + r, c);
+        int k = lane;
+#pragma unroll 4
+        for (; k + 32 < M; k += 64) {
+            const float2 z0 = b.P.load(Z, k, c), z1 = b.P.load(Z, k + 32, c);
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                acc[r] = cfma(vec[r * M + k], z0, acc[r]);
+                acc2[r] = cfma(vec[r * M + k + 32], z1, acc2[r]);
             }
-            if (k < M) acc = cfma(vec[k], P.load(Z, k, c), acc);
-            acc = warp_sum(acc + acc2);
-            if (lane == 0) border_store(O, U, P, us, os, alpha, i, c, acc);
         }
-        __syncthreads();
+        if (k < M) {
+            const float2 z0 = b.P.load(Z, k, c);
+#pragma unroll
+            for (int r = 0; r < NR; ++r) acc[r] = cfma(vec[r * M + k], z0, acc[r]);
+        }
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const float2 s = warp_sum(acc[r] + acc2[r]);
+            if (lane == 0) border_store(b, w, b.R + r, c, s, u[r]);
+        }
     }
-    for (int c = NT; c < M; ++c) {              // border columns: (V zs)[:R, :] Z[:, c]
+}
+
+// Border columns [NT, M) of 64 rows: a column of Z zs and the walker's field
+// table in shared memory, a warp per row.
+__device__ __forceinline__ void border_columns(const BorderArgs& b, float2* vec, int w, int i0) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, M = b.M;
+    const float* Z = b.Zin + b.wstride * w;
+    const float2* ph = b.phi + (size_t)w * b.nslot;
+    float2* phs = vec + M;                                  // [nslot]
+    for (int e = threadIdx.x; e < b.nslot; e += blockDim.x) phs[e] = ph[e];
+    for (int c = b.NT; c < M; ++c) {
+        __syncthreads();
         for (int k = threadIdx.x; k < M; k += blockDim.x) {
-            const ScaleF sk(zs ? zs[k] : 1.0);
-            const float2 z = P.load(Z, k, c);
+            const ScaleF sk(b.first ? b.h[k] : make_float2(1.f, 0.f));
+            const float2 z = b.P.load(Z, k, c);
             vec[k] = make_float2(sk(z.x), sk(z.y));
         }
         __syncthreads();
-        for (int i = warp; i < Rr; i += nw) {
-            const int base = pks[i] + qoff;
+        for (int i = i0 + warp; i < min(b.R, i0 + 64); i += 8) {
+            const uint16_t* row = b.vidx + (size_t)i * M;
+            const float2 u = b.P.load(b.Yu + b.wstride * w, i, c);
             float2 acc = make_float2(0.f, 0.f);
-            for (int k = lane; k < M; k += 32) acc = cfma(phs[qs[base - pks[k]]], vec[k], acc);
+#pragma unroll 4
+            for (int k = lane; k < M; k += 32) acc = cfma(phs[row[k]], vec[k], acc);
             acc = warp_sum(acc);
-            if (lane == 0) border_store(O, U, P, us, os, alpha, i, c, acc);
+            if (lane == 0) border_store(b, w, i, c, acc, u);
         }
-        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(256) k_chain_border(const BorderArgs b, int row_blocks) {
+    extern __shared__ unsigned char smem_raw[];
+    float2* vec = reinterpret_cast<float2*>(smem_raw);
+    const int w = blockIdx.y;
+    if ((int)blockIdx.x >= row_blocks) {
+        border_columns(b, vec, w, ((int)blockIdx.x - row_blocks) * 64);
+        return;
+    }
+    const int c0 = blockIdx.x * BC;
+    switch (b.M - b.R) {
+        case 1: border_rows<1>(b, vec, w, c0); break;
+        case 2: border_rows<2>(b, vec, w, c0); break;
+        case 3: border_rows<3>(b, vec, w, c0); break;
+        case 4: border_rows<4>(b, vec, w, c0); break;
+        case 5: border_rows<5>(b, vec, w, c0); break;
+        case 6: border_rows<6>(b, vec, w, c0); break;
+        case 7: border_rows<7>(b, vec, w, c0); break;
+        default: border_rows<BORDER_ROWS>(b, vec, w, c0); break;
     }
 }
 
@@ -639,12 +682,29 @@ cudaError_t launch_items(ftq_ctx* timing_ctx, TcBatch& tb, const int4* items, in
 cudaError_t launch_border(ftq_ctx* c, const float* zin, float* out, const double* zs, const double* os, float alpha) {
     int R, NT;
     tc_plan(c->M, c->nct, &R, &NT);
-    if (R >= c->M && NT * c->nct >= c->M) return cudaSuccess;
-    Planes P;
-    P.Kp = c->Kp;
-    P.part = (size_t)c->LD * 2 * c->Kp;
-    const int qsize = c->sys.qS * c->sys.qS * c->sys.qS;
-    const size_t bsm = sizeof(float2) * (c->M + c->nslot) + sizeof(int) * c->M + sizeof(uint16_t) * qsize;
+    const bool rows = R < c->M, cols = NT * c->nct < c->M;
+    if (!rows && !cols) return cudaSuccess;
+    BorderArgs b;
+    b.Zin = zin;
+    b.Yu = c->Ypl;
+    b.out = out;
+    b.phi = c->phi32;
+    b.vidx = c->tab.vidx;
+    b.h = c->tab.hf;                      // the only scale the chain uses is h
+    b.alpha = alpha;
+    b.M = c->M;
+    b.nslot = c->nslot;
+    b.R = std::min(R, c->M);
+    b.NT = NT * c->nct;
+    b.first = zs ? 1 : 0;
+    b.last = os ? 1 : 0;
+    b.P.Kp = c->Kp;
+    b.P.part = (size_t)c->LD * 2 * c->Kp;
+    b.wstride = 2 * b.P.part;
+    const int nrow = rows ? (c->M + BC - 1) / BC : 0;
+    const int ncol = cols ? (b.R + 63) / 64 : 0;
+    const size_t bsm = sizeof(float2) * std::max((size_t)(c->M - b.R) * c->M * (rows ? 1 : 0),
+                                                 (size_t)(c->M + c->nslot) * (cols ? 1 : 0));
     static size_t bsm_set = 48 * 1024;
     if (bsm > bsm_set) {
         cudaError_t e = cudaFuncSetAttribute(k_chain_border, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsm);
@@ -652,9 +712,7 @@ cudaError_t launch_border(ftq_ctx* c, const float* zin, float* out, const double
         bsm_set = bsm;
     }
     LaunchScope ls(c, FTQ_K_BORDER);
-    k_chain_border<<<c->W, 256, bsm, c->stream>>>(zin, c->Ypl, out, c->phi, c->tab.pk, c->tab.qcube, zs, c->tab.h, os,
-                                                 alpha, c->M, c->nslot, qsize, c->sys.qoff, P, 2 * P.part, R,
-                                                 NT * c->nct);
+    k_chain_border<<<dim3((unsigned)(nrow + ncol), (unsigned)c->W), 256, bsm, c->stream>>>(b, nrow);
     return cudaGetLastError();
 }
 
