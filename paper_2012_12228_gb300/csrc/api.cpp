@@ -47,7 +47,7 @@ void free_all(ftq_ctx* c) {
                     c->tab.cq, c->tab.vq, c->tab.vqf, c->tab.ksq, c->tab.g0, c->items, c->tab.pk, c->tab.qcube,
                     c->tab.hf, c->phi32, c->xbuf, c->xsum, c->pc_w, c->pc_cnt, c->pc_parent, c->pc_pairs,
                     c->sq_walker, c->sq_w, c->sq_out, c->Yf, c->tab.eplus, c->trk, c->trk_out, c->items_lr,
-                    c->oz_dig, c->oz_ev, c->oz_cmax, c->tab.ozidx, c->lu_scal, c->lu_int};
+                    c->oz_dig, c->oz_ev, c->oz_cmax, c->tab.ozidx, c->lu_scal, c->lu_int, c->est_parts};
     for (void* p : ptrs)
         if (p) cudaFree(p);
 }
@@ -176,6 +176,7 @@ int ftq_init_ueg(ftq_ctx** out, int N, int M, double rs, double theta, double mu
     chk(dalloc(c, &c->pc_parent, W));
     chk(dalloc(c, &c->pc_pairs, 1 + 2 * W));
     chk(dalloc(c, &c->est, W * ftq::WSTRIDE));
+    chk(dalloc(c, &c->est_parts, W * ftq::EST_PARTS * 6));
     chk(dalloc(c, &c->red, 16));
     chk(dalloc(c, &c->status, 1));
     const ftq::UegSetup& s = c->sys;

@@ -9,8 +9,8 @@
 // is the trace of a product of two gathered blocks, tr(XY) = tr(YX)), so only
 // the half-space transfers are summed and counted twice.
 //
-// k_est_walkers: persistent blocks over walkers (a walker's G stays in L2
-// while its block works on it); a warp per slot for rho; for Lambda a warp
+// k_est_walkers: persistent blocks over walkers, or over parts of them when there
+// are fewer walkers than blocks (a walker's G stays in L2 while it is worked on); a warp per slot for rho; for Lambda a warp
 // per work unit = 32 consecutive pairs (a, d) of one +Q transfer (one per
 // lane), looping over all pairs (b, c) of that transfer: P_ab = delta_ab -
 // G[b][a] is read from row b of G and P_cd = delta_cd - G[d][c] from row c
@@ -25,6 +25,7 @@
 
 #include "block_reduce.cuh"
 #include "complex_math.cuh"
+#include "exchange.cuh"
 #include "ftq_internal.h"
 
 namespace ftq {
@@ -41,20 +42,6 @@ __device__ __forceinline__ double2 pel(const double2* Gw, int M, int a, int b) {
 __device__ __forceinline__ float2 pel(const float2* Gw, int M, int a, int b) {
     const float2 g = Gw[(long)b * M + a];
     return make_float2((a == b ? 1.f : 0.f) - g.x, -g.y);
-}
-
-// The delta terms of (delta_1 - g1)(delta_2 - g2) - g1 g2.
-__device__ __forceinline__ double2 delta_terms(bool d1, bool d2, double2 g1, double2 g2) {
-    double2 r = make_double2((d1 && d2) ? 1.0 : 0.0, 0.0);
-    if (d1) r = r - g2;
-    if (d2) r = r - g1;
-    return r;
-}
-__device__ __forceinline__ float2 delta_terms(bool d1, bool d2, float2 g1, float2 g2) {
-    float2 r = make_float2((d1 && d2) ? 1.f : 0.f, 0.f);
-    if (d1) r = r - g2;
-    if (d2) r = r - g1;
-    return r;
 }
 
 // Gt[w] = G[w]^T through 32 x 33 shared tiles; grid (tiles, tiles, W).
@@ -88,16 +75,18 @@ __global__ void __launch_bounds__(1024) k_est_walkers(const T* __restrict__ G, c
                                                     int nunits, const double* __restrict__ vq,
                                                     const float2* __restrict__ vqf,
                                                     const double* __restrict__ ksq, int M, int nqh, double E_M,
-                                                    int W) {
+                                                    int W, int nparts, double* __restrict__ parts) {
     extern __shared__ unsigned char smem_raw[];
     double2* rho = reinterpret_cast<double2*>(smem_raw);     // [2 nqh + 1]
     __shared__ double2 shc[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int nslot = 2 * nqh + 1;
-    for (int w = blockIdx.x; w < W; w += gridDim.x) {
+    for (int item = blockIdx.x; item < W * nparts; item += gridDim.x) {
+        const int w = item / nparts, part = item % nparts;
         const T* Gw = G + (size_t)w * M * M;
         const T* Gt = Gtr + (size_t)w * M * M;
-        for (int sl = 1 + warp; sl < nslot; sl += nw) {
+        // the first part of a walker also takes everything but the exchange sum
+        for (int sl = 1 + warp; sl < nslot && part == 0; sl += nw) {
             double2 r = make_double2(0.0, 0.0);
             for (int e = pptr[sl] + lane; e < pptr[sl + 1]; e += 32) r = r + to_d(pel(Gw, M, pa[e], pb[e]));
             r = warp_sum_d(r);
@@ -108,44 +97,17 @@ __global__ void __launch_bounds__(1024) k_est_walkers(const T* __restrict__ G, c
         // FP32 G: v_Q acc accumulated per lane as a compensated float sum
         // (hi + lo, two-sum), so that no FP64 instruction runs per pair
         float exh[2] = {0.f, 0.f}, exl[2] = {0.f, 0.f};
-        for (int a = threadIdx.x; a < M; a += blockDim.x) {
+        for (int a = threadIdx.x; a < M && part == 0; a += blockDim.x) {
             const double2 p = to_d(pel(Gw, M, a, a));
             nsum = nsum + p * 2.0;
             e1 = e1 + p * ksq[a];
         }
-        for (int q = threadIdx.x; q < nqh; q += blockDim.x) e2 = e2 + cmul(rho[1 + 2 * q], rho[2 + 2 * q]) * (4.0 * vq[q]);
-        for (int u = warp; u < nunits; u += nw) {
+        for (int q = threadIdx.x; q < nqh && part == 0; q += blockDim.x) e2 = e2 + cmul(rho[1 + 2 * q], rho[2 + 2 * q]) * (4.0 * vq[q]);
+        for (int u = warp * nparts + part; u < nunits; u += nw * nparts) {
             const int4 un = units[u];                  // slot pairs [x, y), chunk from z, v_Q index w
             const int f = un.z + lane;
             const bool on = f < un.y;
-            const int al = on ? pa[f] : 0, dl = on ? pb[f] : 0;
-            const T* gcol = Gw + al;                   // G[b][al] = gcol[b * M]
-            const T* tcol = Gt + dl;                   // G[dl][c] = G^T[c][dl] = tcol[c * M]
-            // P_ab P_cd = (delta_ab - g1)(delta_cd - g2) with g1 = G[b][a],
-            // g2 = G[d][c]: the product g1 g2 every time, the delta terms
-            // only where an index matches (once per lane and unit at most)
-            T acc, acc2;
-            acc.x = 0;
-            acc.y = 0;
-            acc2 = acc;
-            int g = un.x;
-#pragma unroll 1
-            for (; g + 1 < un.y; g += 2) {
-                const int b0 = pa[g], c0 = pb[g], b1 = pa[g + 1], c1 = pb[g + 1];   // the same for every lane
-                const T x0 = gcol[(size_t)b0 * M], y0 = tcol[(size_t)c0 * M];
-                const T x1 = gcol[(size_t)b1 * M], y1 = tcol[(size_t)c1 * M];
-                acc = cfma(x0, y0, acc);
-                acc2 = cfma(x1, y1, acc2);
-                if (al == b0 || c0 == dl) acc = acc + delta_terms(al == b0, c0 == dl, x0, y0);
-                if (al == b1 || c1 == dl) acc2 = acc2 + delta_terms(al == b1, c1 == dl, x1, y1);
-            }
-            if (g < un.y) {
-                const int b0 = pa[g], c0 = pb[g];
-                const T x0 = gcol[(size_t)b0 * M], y0 = tcol[(size_t)c0 * M];
-                acc = cfma(x0, y0, acc);
-                if (al == b0 || c0 == dl) acc = acc + delta_terms(al == b0, c0 == dl, x0, y0);
-            }
-            acc = acc + acc2;
+            const T acc = exchange_unit<T>(Gw, Gt, M, pa, pb, un.x, un.y, on ? pa[f] : 0, on ? pb[f] : 0);
             if (!on) continue;
             const int qi = un.w;
             if constexpr (sizeof(T) == sizeof(float2)) {
@@ -171,7 +133,10 @@ __global__ void __launch_bounds__(1024) k_est_walkers(const T* __restrict__ G, c
         nsum = block_sum(nsum, shc);
         e1 = block_sum(e1, shc);
         e2 = block_sum(e2, shc);
-        if (threadIdx.x == 0) {
+        if (threadIdx.x == 0 && nparts > 1) {
+            double* o = parts + 6 * (size_t)item;
+            o[0] = e1.x; o[1] = e1.y; o[2] = e2.x; o[3] = e2.y; o[4] = nsum.x; o[5] = nsum.y;
+        } else if (threadIdx.x == 0) {
             const double* s = ws + (long)WSTRIDE * w;
             double* o = est + (long)WSTRIDE * w;
             o[0] = s[0]; o[1] = s[1]; o[2] = s[2];
@@ -179,6 +144,21 @@ __global__ void __launch_bounds__(1024) k_est_walkers(const T* __restrict__ G, c
             o[5] = nsum.x; o[6] = nsum.y; o[7] = 0.0;
         }
     }
+}
+
+// The parts of every walker summed in order.
+__global__ void k_est_combine(const double* __restrict__ parts, const double* __restrict__ ws,
+                              double* __restrict__ est, int W, int nparts, double E_M) {
+    const int w = blockIdx.x * blockDim.x + threadIdx.x;
+    if (w >= W) return;
+    double v[6] = {};
+    for (int q = 0; q < nparts; ++q)
+        for (int k = 0; k < 6; ++k) v[k] += parts[6 * ((size_t)w * nparts + q) + k];
+    const double* s = ws + (long)WSTRIDE * w;
+    double* o = est + (long)WSTRIDE * w;
+    o[0] = s[0]; o[1] = s[1]; o[2] = s[2];
+    o[3] = E_M + v[0] + v[2]; o[4] = v[1] + v[3];
+    o[5] = v[4]; o[6] = v[5]; o[7] = 0.0;
 }
 
 // sum_w of w, wE, wN with w = exp(ln|w| - s) e^{i arg w}, s = max ln|w| over
@@ -248,6 +228,12 @@ __global__ void k_slice_summary(const double* __restrict__ rec, int n, double* _
 }
 
 template <typename T>
+void transpose_g(ftq_ctx* c, const T* G, T* Gt) {
+    const unsigned tiles = (unsigned)((c->M + 31) / 32);
+    k_transpose_g<T><<<dim3(tiles, tiles, (unsigned)c->W), dim3(32, 8), 0, c->stream>>>(G, Gt, c->M);
+}
+
+template <typename T>
 cudaError_t launch_est_walkers(ftq_ctx* c, const T* G) {
     const int nqh = c->sys.nq_half;
     const int M = c->M;
@@ -268,21 +254,34 @@ cudaError_t launch_est_walkers(ftq_ctx* c, const T* G) {
     // the L2; complex128 G (FP64-pipe bound): two 512-thread blocks per SM
     const int nthr = f32 ? 1024 : 512;
     const int per_sm = f32 ? 1 : 2;
-    const int grid = c->W < per_sm * sms ? c->W : per_sm * sms;
+    // fewer walkers than four rounds of blocks (FP32 G: than blocks, since the loads of a
+    // split walker's G come from L2 more than once): a walker's exchange units are split
+    // (M = 257, 128 walkers, complex128: 5.8 ms with one block each, 5.0 split)
+    const int target = f32 ? sms : 4 * per_sm * sms;
+    int nparts = c->W < target ? (target + c->W - 1) / c->W : 1;
+    nparts = nparts > EST_PARTS ? EST_PARTS : nparts;
+    const int grid = c->W * nparts < per_sm * sms ? c->W * nparts : per_sm * sms;
     LaunchScope ls(c, FTQ_K_ESTIMATORS);
     // G^T into the complex128 work buffer (scratch between calls; it holds a
     // complex128 or a complex64 matrix per walker)
     T* Gt = reinterpret_cast<T*>(c->work);
-    const int tiles = (M + 31) / 32;
-    k_transpose_g<T><<<dim3((unsigned)tiles, (unsigned)tiles, (unsigned)c->W), dim3(32, 8), 0, c->stream>>>(G, Gt, M);
+    transpose_g(c, G, Gt);
     c->launches[FTQ_K_ESTIMATORS] += 1;
     k_est_walkers<T><<<grid, nthr, sm, c->stream>>>(G, Gt, c->wstate, c->est, c->tab.pair_ptr, c->tab.pair_a,
                                                     c->tab.pair_b, c->tab.vidx, c->tab.eplus, c->tab.neplus,
-                                                    c->tab.vq, c->tab.vqf, c->tab.ksq, M, nqh, c->sys.E_M, c->W);
+                                                    c->tab.vq, c->tab.vqf, c->tab.ksq, M, nqh, c->sys.E_M, c->W,
+                                                    nparts, c->est_parts);
+    if (nparts > 1) {
+        c->launches[FTQ_K_ESTIMATORS] += 1;
+        k_est_combine<<<(c->W + 127) / 128, 128, 0, c->stream>>>(c->est_parts, c->wstate, c->est, c->W, nparts,
+                                                              c->sys.E_M);
+    }
     return cudaGetLastError();
 }
 
 }  // namespace
+
+void launch_transpose_g(ftq_ctx* c, const double2* G, double2* Gt) { transpose_g(c, G, Gt); }
 
 cudaError_t launch_estimators(ftq_ctx* c, double* per_walker) {
     if (!c->g64_valid) {

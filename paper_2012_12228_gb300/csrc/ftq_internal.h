@@ -19,6 +19,7 @@ namespace ftq {
 //   [0..2] as above, [3] Re E, [4] Im E, [5] Re N, [6] Im N, [7] unused,
 //   [8] d ln|w|/dmu, [9] d arg w/dmu, [10] Re dE, [11] Im dE, [12] Re dN, [13] Im dN
 constexpr int WSTRIDE = 16;
+constexpr int EST_PARTS = 8;      // most blocks that share a walker's estimators
 
 // Static description of one UEG system (Sec. "Uniform Electron Gas" and
 // "Computational Details").  Built on the host once per context.
@@ -146,6 +147,7 @@ struct ftq_ctx {
     int* perm = nullptr;          // pivot permutation scratch                 [W][M]
     double* wstate = nullptr;     // [W][WSTRIDE] per-walker state (layout above)
     double* est = nullptr;        // [W][WSTRIDE] per-walker estimators
+    double* est_parts = nullptr;  // [W][EST_PARTS][6] partial sums of the estimators
     double* red = nullptr;        // [16] reduced sums (estimators, mu derivative)
     // time-slice estimates: every track_every-th slice, records {k, E_k, N_k, alive, sum w, scale}
     int track_every = 0;
@@ -212,6 +214,7 @@ cudaError_t launch_chain(ftq_ctx* c);
 cudaError_t launch_qrcp(ftq_ctx* c);
 cudaError_t launch_green(ftq_ctx* c, int k, bool update_weights);
 cudaError_t launch_estimators(ftq_ctx* c, double* per_walker);
+void launch_transpose_g(ftq_ctx* c, const double2* G, double2* Gt);
 // Estimators of slice k into the next slice record (estimators.cu).
 cudaError_t launch_slice_estimate(ftq_ctx* c, int k);
 cudaError_t launch_slice_summary(ftq_ctx* c, double* out_dev, int rows);

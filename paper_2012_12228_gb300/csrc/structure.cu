@@ -5,9 +5,11 @@
 // Gamma_Q = (2 rho_Q)(2 rho_-Q), Lambda_Q = 2 sum_{K1 K2} P_{K1+Q,K2} P_{K2-Q,K1}
 // (the exchange sum of the energy estimator) and
 // D_Q = 2 sum_{K: K, K+Q in basis} P_{K+Q,K+Q}.
+#include <algorithm>
 #include <cmath>
 
 #include "complex_math.cuh"
+#include "exchange.cuh"
 #include "ftq_internal.h"
 
 namespace ftq {
@@ -15,44 +17,57 @@ namespace {
 
 // P_ab = <a+_a a_b> = delta_ab - G_ba
 __device__ __forceinline__ double2 pel_s(const double2* Gw, int M, int a, int b) {
-    const double2 g = Gw[(long)b * M + a];
+    const double2 g = Gw[(size_t)b * M + a];
     return make_double2((a == b ? 1.0 : 0.0) - g.x, -g.y);
 }
 
-// One block per walker; slot sl (1 .. nslot-1) is the transfer of the pair
-// lists (odd: +q of the half space, even: -q).
-__global__ void k_structure(const double2* __restrict__ G, const int* __restrict__ pptr,
-                            const int* __restrict__ pa, const int* __restrict__ pb,
-                            const uint16_t* __restrict__ vidx, double2* __restrict__ out, int M, int nslot) {
-    extern __shared__ unsigned char smem_raw[];
-    double2* rho = reinterpret_cast<double2*>(smem_raw);    // [nslot]
-    double2* acc = rho + nslot;                             // [nslot]: D_Q - Lambda_Q
-    const int w = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
-    const double2* Gw = G + (long)w * M * M;
-    for (int sl = 1 + tid; sl < nslot; sl += nt) {
-        double2 r = make_double2(0.0, 0.0), d = make_double2(0.0, 0.0);
-        for (int e = pptr[sl]; e < pptr[sl + 1]; ++e) {
-            r = r + pel_s(Gw, M, pa[e], pb[e]);
-            d = d + pel_s(Gw, M, pa[e], pa[e]);
+__device__ __forceinline__ double2 warp_total(double2 v) {
+    for (int o = 16; o > 0; o >>= 1) {
+        v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+        v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+    }
+    return v;
+}
+
+// A warp per walker and half-space transfer q (slots 1 + 2 q and 2 + 2 q, whose
+// pairs are each other's reversed): rho and D of both, and Lambda once, since
+// Lambda_-Q = Lambda_Q.  The short transfers have the most pairs and come first;
+// the warps of a walker's blocks take them in turn.  The FP64 pipe bounds it (four
+// DFMA per exchange term).
+__global__ void __launch_bounds__(512) k_structure(const double2* __restrict__ G, const double2* __restrict__ Gtr,
+                                                  const int* __restrict__ pptr, const int* __restrict__ pa,
+                                                  const int* __restrict__ pb, double2* __restrict__ out, int M,
+                                                  int nqh) {
+    const int w = blockIdx.y, lane = threadIdx.x & 31;
+    const int warp = blockIdx.x + gridDim.x * (threadIdx.x >> 5), nw = gridDim.x * (blockDim.x >> 5);
+    const double2* Gw = G + (size_t)w * M * M;
+    const double2* Gt = Gtr + (size_t)w * M * M;
+    for (int q = warp; q < nqh; q += nw) {
+        const int first = pptr[1 + 2 * q], end = pptr[2 + 2 * q];
+        double2 rp = make_double2(0.0, 0.0), rm = rp, dp = rp, dm = rp, lam = rp;
+        for (int e0 = first; e0 < end; e0 += 32) {
+            const int e = e0 + lane;
+            const bool on = e < end;
+            const int a = on ? pa[e] : 0, d = on ? pb[e] : 0;
+            const double2 x = exchange_unit<double2>(Gw, Gt, M, pa, pb, first, end, a, d);
+            if (on) {
+                lam = lam + x;
+                rp = rp + pel_s(Gw, M, a, d);
+                rm = rm + pel_s(Gw, M, d, a);
+                dp = dp + pel_s(Gw, M, a, a);
+                dm = dm + pel_s(Gw, M, d, d);
+            }
         }
-        rho[sl] = r;
-        acc[sl] = d * 2.0;
-    }
-    __syncthreads();
-    const int npair = pptr[nslot];
-    for (int e = tid; e < npair; e += nt) {
-        const int a = pa[e], d = pb[e];
-        const int sl = vidx[(long)a * M + d];
-        double2 lam = make_double2(0.0, 0.0);
-        for (int f = pptr[sl]; f < pptr[sl + 1]; ++f) lam = cfma(pel_s(Gw, M, a, pa[f]), pel_s(Gw, M, pb[f], d), lam);
-        atomicAdd(&acc[sl].x, -2.0 * lam.x);
-        atomicAdd(&acc[sl].y, -2.0 * lam.y);
-    }
-    __syncthreads();
-    for (int sl = 1 + tid; sl < nslot; sl += nt) {
-        const int partner = (sl & 1) ? sl + 1 : sl - 1;
-        const double2 gam = cmul(rho[sl] * 2.0, rho[partner] * 2.0);
-        out[(long)w * (nslot - 1) + sl - 1] = gam + acc[sl];
+        lam = warp_total(lam);
+        rp = warp_total(rp);
+        rm = warp_total(rm);
+        dp = warp_total(dp);
+        dm = warp_total(dm);
+        if (lane == 0) {
+            const double2 g = cmul(rp * 2.0, rm * 2.0) - lam * 2.0;
+            out[((size_t)w * nqh + q) * 2] = g + dp * 2.0;
+            out[((size_t)w * nqh + q) * 2 + 1] = g + dm * 2.0;
+        }
     }
 }
 
@@ -117,6 +132,7 @@ __global__ void k_struct_reduce(const double2* __restrict__ wr, const double2* _
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= nq) return;
     double2 acc = make_double2(0.0, 0.0);
+#pragma unroll 8
     for (int w = 0; w < W; ++w) acc = cfma(wr[w], pw[(long)w * nq + j], acc);
     out[4 + 2 * j] = acc.x;
     out[5 + 2 * j] = acc.y;
@@ -137,15 +153,18 @@ cudaError_t launch_structure_factor(ftq_ctx* c, double* per_walker_out) {
         e = mixed_sync_g64(c);
         if (e != cudaSuccess) return e;
     }
-    const size_t sm = 2 * sizeof(double2) * (size_t)nslot;
-    if (sm > 48 * 1024) {
-        e = cudaFuncSetAttribute(k_structure, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-    }
     {
+        // enough 512-thread blocks for four rounds of two per SM (M = 257, 128 walkers: one 256-thread
+        // block per walker with both signs of Q summed took 14.6 ms)
+        int dev = 0, sms = 1;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        const int per = std::max(1, std::min((8 * sms + W - 1) / W, (nq / 2 + 15) / 16));
         LaunchScope ls(c, FTQ_K_ESTIMATORS);
-        k_structure<<<W, 256, sm, c->stream>>>(c->G, c->tab.pair_ptr, c->tab.pair_a, c->tab.pair_b, c->tab.vidx,
-                                              c->sq_walker, c->M, nslot);
+        c->launches[FTQ_K_ESTIMATORS] += 1;
+        launch_transpose_g(c, c->G, c->work);
+        k_structure<<<dim3((unsigned)per, (unsigned)W), 512, 0, c->stream>>>(c->G, c->work, c->tab.pair_ptr, c->tab.pair_a,
+                                                                         c->tab.pair_b, c->sq_walker, c->M, nq / 2);
     }
     {
         LaunchScope ls(c, FTQ_K_ESTIMATORS);
