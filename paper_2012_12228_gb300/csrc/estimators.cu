@@ -260,6 +260,7 @@ cudaError_t launch_est_walkers(ftq_ctx* c, const T* G) {
     const int target = f32 ? sms : 4 * per_sm * sms;
     int nparts = c->W < target ? (target + c->W - 1) / c->W : 1;
     nparts = nparts > EST_PARTS ? EST_PARTS : nparts;
+    if (nparts > c->tab.neplus / 64) nparts = c->tab.neplus < 64 ? 1 : c->tab.neplus / 64;   // small bases: one block
     const int grid = c->W * nparts < per_sm * sms ? c->W * nparts : per_sm * sms;
     LaunchScope ls(c, FTQ_K_ESTIMATORS);
     // G^T into the complex128 work buffer (scratch between calls; it holds a
