@@ -131,7 +131,7 @@ __global__ void k_qrcp(const double2* __restrict__ Yin, double2* __restrict__ Qo
                        double2* __restrict__ work, double2* __restrict__ work2,
                        double2* __restrict__ DR, double2* __restrict__ Tinv,
                        double2* __restrict__ hh, double* __restrict__ htau,
-                       double* __restrict__ ws, int* __restrict__ status, int M) {
+                       double* __restrict__ ws, int* __restrict__ status, int* __restrict__ perm_out, int M) {
     extern __shared__ unsigned char smem_raw[];
     double* cn = reinterpret_cast<double*>(smem_raw);          // column norms [M]
     int* perm = reinterpret_cast<int*>(cn + M);                 // [M]
@@ -224,6 +224,14 @@ __global__ void k_qrcp(const double2* __restrict__ Yin, double2* __restrict__ Qo
             for (int r = j + 1; r < M; ++r) Q[(long)r * M + c] = cfms(C[(long)r * M + j], s, Q[(long)r * M + c]);
         }
         __syncthreads();
+    }
+    if (perm_out) {                          // T^-1 is updated from R by the kernels of green_lu.cu
+        for (int j = threadIdx.x; j < M; j += nt) perm_out[(long)w * M + j] = perm[j];
+        if (threadIdx.x == 0) {
+            double* s = ws + (long)WSTRIDE * w;
+            s[7] = (double)(((int)s[7]) ^ nswap);
+        }
+        return;
     }
     // D = diag R; U = D^-1 R (strict upper part scaled in place)
     for (int j = threadIdx.x; j < M; j += nt) DR[(long)w * M + j] = C[(long)j * M + j];
@@ -421,10 +429,14 @@ cudaError_t launch_qrcp64(ftq_ctx* c, const double2* Yin, double2* Qout) {
     const int M = c->M;
     size_t sm = sizeof(double) * M + sizeof(int) * M;
     int nt = fact_threads(M);
+    const bool lu = lu64_supported(M);
+    double2* R = lu ? c->zbuf[1] : c->work;      // S of the T^-1 update takes the work buffer
     LaunchScope ls(c, FTQ_K_QRCP);
-    k_qrcp<<<c->W, nt, sm, c->stream>>>(Yin, Qout, c->work, c->work2, c->DR, c->Tinv, c->hh, c->htau,
-                                       c->wstate, c->status, M);
-    return cudaGetLastError();
+    k_qrcp<<<c->W, nt, sm, c->stream>>>(Yin, Qout, R, c->work2, c->DR, c->Tinv, c->hh, c->htau,
+                                       c->wstate, c->status, lu ? c->perm : nullptr, M);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess && lu) e = launch_tinv_lu64(c, R, c->perm);
+    return e;
 }
 
 cudaError_t launch_qrcp(ftq_ctx* c) {

@@ -274,6 +274,8 @@ size_t lu_scal_doubles(int M, int W);
 size_t lu_ints(int W);
 bool lu64_supported(int M);
 cudaError_t lu_make_maps(ftq_ctx* c);
+cudaError_t launch_tinv_lu32(ftq_ctx* c);
+cudaError_t launch_tinv_lu64(ftq_ctx* c, const double2* R, const int* perm);
 cudaError_t launch_green_lu64(ftq_ctx* c, const double2* Y, int k, bool update, bool physical);
 cudaError_t launch_green_lu32(ftq_ctx* c, int k, float2* G = nullptr, double* ws = nullptr);
 

@@ -25,6 +25,7 @@
 #include <cmath>
 
 #include "complex_math.cuh"
+#include "df_math.cuh"
 #include "digits.cuh"
 #include "ftq_internal.h"
 #include "green_tail.cuh"
@@ -112,21 +113,13 @@ __global__ void __launch_bounds__(256) k_lu_form64(const double2* __restrict__ Y
     }
 }
 
-// t s for FP64 t and s = b r in FP32 pairs: the upper 24 bits of t and the rest
-// against the product and its rounding error, about 2^-24 relative in all.  It is
+// t s for FP64 t and s = b r in FP32 pairs, about 2^-24 relative in all.  It is
 // integer and FP32 work only: with three FP64 multiplications and four
 // conversions per entry the kernel ran at the FP64 pipe's rate (1.09 ms at
 // M = 257, 1024 walkers).
 __device__ __forceinline__ float scaled(double t, float sh, float sl) {
-    const int hi = __double2hiint(t);
-    const uint32_t lo = (uint32_t)__double2loint(t);
-    const int e = ((hi >> 20) & 0x7ff) - 1023;
-    if ((((uint32_t)hi << 1) | lo) == 0u) return 0.f;
-    if (e < -70 || e > 126) return (float)(t * ((double)sh + (double)sl));
-    const uint32_t sign = (uint32_t)hi & 0x80000000u;
-    const float th = __uint_as_float(sign | (uint32_t)(e + 127) << 23 | ((uint32_t)hi & 0xfffffu) << 3 | lo >> 29);
-    const float tl = (float)(int)(lo & 0x1fffffffu) * __uint_as_float(sign | (uint32_t)(e - 52 + 127) << 23);
-    return fmaf(th, sh, fmaf(th, sl, tl * sh));
+    const df2 v = df_split_int(t);
+    return fmaf(v.h, sh, fmaf(v.h, sl, v.l * sh));
 }
 
 // The same from the FP32 planes, whose columns are contiguous along c here.
@@ -250,7 +243,7 @@ __global__ void __launch_bounds__(MAXT) k_lu_panel(cx<T>* __restrict__ S, LuScal
 // ---------------------------------------------------------------- triangles
 // One column of S per thread.  Forward: the panel's permutation on its rows,
 // then X <- L11^-1 X.  Backward: X <- U11^-1 X.
-template <typename T, int NB, bool UPPER>
+template <typename T, int NB, bool UPPER, bool PERM = !UPPER>
 __global__ void __launch_bounds__(128) k_lu_tri(cx<T>* __restrict__ S, LuScales<T> sc, int M, int ld, int jb, int nb,
                                                int cbeg, int cend) {
     __shared__ cx<T> D[NB][NB];
@@ -264,7 +257,8 @@ __global__ void __launch_bounds__(128) k_lu_tri(cx<T>* __restrict__ S, LuScales<
         D[r][c] = r < nb && c < nb ? Sw[(size_t)(jb + r) * ld + jb + c] : mk<T>(0, 0);
     }
     for (int q = tid; q < NB; q += nt) {
-        inv[q] = q < nb ? sc.inv[(size_t)w * M + jb + q] : mk<T>(0, 0);
+        if (UPPER) inv[q] = q < nb ? sc.inv[(size_t)w * M + jb + q] : mk<T>(0, 0);
+        if (!PERM) continue;
         src[q] = q < nb ? sc.perm[(size_t)w * 2 * LU_NB_MAX + q] : 0;
         dst[q] = q < nb ? sc.perm[(size_t)w * 2 * LU_NB_MAX + LU_NB_MAX + q] : -1;
     }
@@ -274,9 +268,9 @@ __global__ void __launch_bounds__(128) k_lu_tri(cx<T>* __restrict__ S, LuScales<
     cx<T>* col = Sw + (size_t)jb * ld + c;
     cx<T> x[NB];
 #pragma unroll
-    for (int q = 0; q < NB; ++q) x[q] = q < nb ? col[(size_t)(UPPER ? q : src[q]) * ld] : mk<T>(0, 0);
+    for (int q = 0; q < NB; ++q) x[q] = q < nb ? col[(size_t)(PERM ? src[q] : q) * ld] : mk<T>(0, 0);
     if constexpr (!UPPER) {
-        for (int q = 0; q < nb; ++q)
+        for (int q = 0; PERM && q < nb; ++q)
             if (dst[q] >= 0) col[(size_t)dst[q] * ld] = col[(size_t)q * ld];
 #pragma unroll
         for (int q = 1; q < NB; ++q) {
@@ -299,11 +293,53 @@ __global__ void __launch_bounds__(128) k_lu_tri(cx<T>* __restrict__ S, LuScales<
         if (q < nb) col[(size_t)q * ld] = x[q];
 }
 
+// The forward triangle of the T^-1 update (unit lower, no permutation) with the
+// arithmetic of the mixed path's stabilisation: double-FP32 (48 bits) on the FP32
+// pipe, whose rate is 64 times that of the FP64 pipe.  One column per thread, kept in
+// shared memory ([32][threads] of Re hi, Re lo, Im hi, Im lo), so that the loops stay
+// rolled: 48 instructions per complex term would not fit the instruction cache.
+__global__ void __launch_bounds__(128) k_tinv_tri_df(double2* __restrict__ S, int M, int ld, int jb, int nb, int cbeg,
+                                                    int cend) {
+    extern __shared__ unsigned char smem_raw[];
+    float4* D = reinterpret_cast<float4*>(smem_raw);         // [32][32]
+    float4* X = D + 32 * 32;                                 // [32][threads]
+    const int w = blockIdx.y, tid = threadIdx.x, nt = blockDim.x;
+    double2* Sw = S + (size_t)w * M * ld;
+    for (int e = tid; e < 32 * 32; e += nt) {
+        const int r = e >> 5, c = e & 31;
+        if (r < nb && c < r) {
+            const double2 v = Sw[(size_t)(jb + r) * ld + jb + c];
+            const df2 re = df_split_int(v.x), im = df_split_int(v.y);
+            D[e] = make_float4(re.h, re.l, im.h, im.l);
+        }
+    }
+    __syncthreads();
+    const int c = cbeg + blockIdx.x * nt + tid;
+    if (c >= cend) return;
+    double2* col = Sw + (size_t)jb * ld + c;
+    float4* x = X + tid;
+    for (int q = 0; q < nb; ++q) {
+        const double2 v = col[(size_t)q * ld];
+        df2 re = df_split_int(v.x), im = df_split_int(v.y);
+#pragma unroll 4
+        for (int k = 0; k < q; ++k) {
+            const float4 u = D[q * 32 + k], y = x[k * nt];
+            df_msub(re, y.x, y.y, u.x, u.y);                 // s -= x u
+            df_madd(re, y.z, y.w, u.z, u.w);
+            df_msub(im, y.x, y.y, u.z, u.w);
+            df_msub(im, y.z, y.w, u.x, u.y);
+        }
+        re = df_norm(re);
+        im = df_norm(im);
+        x[q * nt] = make_float4(re.h, re.l, im.h, im.l);
+        col[(size_t)q * ld] = make_double2((double)re.h + (double)re.l, (double)im.h + (double)im.l);
+    }
+}
+
 // ---------------------------------------------------------------- updates
 // C[r0.., c0..) -= S[r, jb .. jb + nb) S[jb .. jb + nb, c] on the tensor cores.
-// Work item = (walker, 64 rows, OCT columns); warps 0..7 epilogue (two per TMEM
-// lane quadrant, half of the columns each; C tiles come and go by TMA, one item
-// ahead: per-thread copies took 60% of an item's time), 8..15
+// Work item = (walker, 64 rows, OCT columns); warps 0..7 epilogue (two groups, C
+// tiles come and go by TMA: per-thread copies took 60% of an item's time), 8..15
 // operand A, 16..19 operand B, 20 control.  Complex as real:
 // MMA rows 2 i = Re, 2 i + 1 = Im of row i (so that a warp's lanes hold whole complex
 // numbers of 16 rows and meet no bank conflicts in the C tile) and k tiles
@@ -395,7 +431,7 @@ __global__ void __launch_bounds__(NT_UP, 1) k_lu_update(const UpArgs<T> p, const
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&tfull[b], 1);
-            mbar_init(&tempty[b], W_EPI);
+            mbar_init(&tempty[b], W_EPI / 2);
             mbar_init(&einfo[b], W_A + W_B);
             mbar_init(&cfull[b], 1);
         }
@@ -614,7 +650,10 @@ __global__ void __launch_bounds__(NT_UP, 1) k_lu_update(const UpArgs<T> p, const
         }
     } else {
         // ------------------------------------------------ epilogue
-        const int quad = warp & 3, half = warp >> 2;         // TMEM lanes, columns
+        // Two groups of four warps (one per TMEM lane quadrant) take the items in turn, each
+        // with its accumulator and its C buffer, so that one group's waits and copies pass
+        // under the other's arithmetic (the FP64 pipe bounds the complex128 items).
+        const int grp = warp >> 2, quad = warp & 3;
         const int part = lane & 1, rr = quad * 16 + (lane >> 1);
         // column of a chunk of 8 that this lane handles q-th: rows that share banks differ in it
         auto at = [&](int q) { return (q + rr) & 7; };
@@ -627,33 +666,34 @@ __global__ void __launch_bounds__(NT_UP, 1) k_lu_update(const UpArgs<T> p, const
             col0 = p.c0 + (tile % p.nct) * OCT;
             boxes = (min(64, p.r1 - row0) + CBOX - 1) / CBOX;
         };
-        // one thread moves the C tiles (rows beyond M and columns beyond ld are the map's business)
-        const bool mover = warp == 0 && lane == 0;
-        auto fetch = [&](int it, int b) {
-            tile_at(it);
-            mbar_expect_tx(&cfull[b], (uint32_t)(boxes * CBOX * CROW));
+        // one thread of the group moves its C tiles (rows beyond M and columns beyond ld are the map's business)
+        const bool mover = quad == 0 && lane == 0;
+        unsigned char* cbuf = ctile + (size_t)grp * 64 * CROW;
+        auto fetch = [&]() {
+            mbar_expect_tx(&cfull[grp], (uint32_t)(boxes * CBOX * CROW));
             for (int q = 0; q < boxes; ++q)
-                tma_load_3d(ctile + (size_t)(b * 64 + q * CBOX) * CROW, &map, col0 * XF, row0 + q * CBOX, w, &cfull[b]);
+                tma_load_3d(cbuf + (size_t)q * CBOX * CROW, &map, col0 * XF, row0 + q * CBOX, w, &cfull[grp]);
         };
-        if (mover && it0 < it1) fetch(it0, 0);
-        for (int it = it0, li = 0; it < it1; ++it, ++li) {
-            const int bi = li & 1;
-            if (mover && it + 1 < it1) {
-                bulk_wait_read();                            // the tile stored from the other buffer has left it
-                fetch(it + 1, bi ^ 1);
+        unsigned char* ct = cbuf + (size_t)rr * CROW + part * sizeof(T);
+        const int bi = grp;
+        int own = 0;                                         // items of this group so far
+        for (int it = it0 + grp; it < it1; it += 2, ++own) {
+            tile_at(it);
+            if (mover) {
+                if (own > 0) bulk_wait_read();               // the tile stored before has left the buffer
+                fetch();
             }
             __syncwarp();
-            tile_at(it);
-            unsigned char* ct = ctile + (size_t)(bi * 64 + rr) * CROW + part * sizeof(T);
-            bool ok = wait(&tfull[bi], (uint32_t)((li >> 1) & 1));
-            ok = ok && wait(&cfull[bi], (uint32_t)((li >> 1) & 1));
-            if constexpr (F64) ok = ok && wait(&einfo[bi], (uint32_t)((li >> 1) & 1));
+            const uint32_t ph = (uint32_t)(own & 1);
+            bool ok = wait(&tfull[bi], ph);
+            ok = ok && wait(&cfull[bi], ph);
+            if constexpr (F64) ok = ok && wait(&einfo[bi], ph);
             tc_fence_after();
             if (ok) {
                 const uint32_t acc = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(bi * ND * OCT);
                 const int er = F64 ? row_e[bi][rr] : 0;
 #pragma unroll 1
-                for (int cc = half * (OCT / 2); cc < (half + 1) * (OCT / 2); cc += 8) {
+                for (int cc = 0; cc < OCT; cc += 8) {
                     if (col0 + cc >= p.c1) break;
                     uint32_t v[ND][8];
 #pragma unroll
@@ -711,17 +751,16 @@ __global__ void __launch_bounds__(NT_UP, 1) k_lu_update(const UpArgs<T> p, const
             fence_async_smem();
             __syncwarp();
             if (lane == 0) mbar_arrive(&tempty[bi]);
-            asm volatile("bar.sync 3, %0;" ::"n"(32 * W_EPI) : "memory");
+            asm volatile("bar.sync %0, %1;" ::"r"(3 + grp), "n"(16 * W_EPI) : "memory");
             if (mover && ok) {
                 for (int q = 0; q < boxes; ++q)
-                    tma_store_3d(ctile + (size_t)(bi * 64 + q * CBOX) * CROW, &map, col0 * XF, row0 + q * CBOX, w);
+                    tma_store_3d(cbuf + (size_t)q * CBOX * CROW, &map, col0 * XF, row0 + q * CBOX, w);
                 bulk_commit();
             }
         }
-        if (mover) {
-            // after an abort a fetched tile may not have been waited for: it must land before the block ends
-            const int n = it1 - it0;
-            for (int li = max(0, n - 2); li < n; ++li) mbar_wait(&cfull[li & 1], (uint32_t)((li >> 1) & 1));
+        if (mover && own > 0) {
+            // after an abort the last tile may not have been waited for: it must land before the block ends
+            mbar_wait(&cfull[grp], (uint32_t)((own - 1) & 1));
             bulk_wait();
         }
     }
@@ -787,8 +826,99 @@ __global__ void __launch_bounds__(128) k_lu_tail(const cx<T>* __restrict__ S, co
     }
 }
 
+// ---------------------------------------------------------------- T^-1 <- T^-1 Pi U^-1
+// X U = Z (Z = T^-1 Pi) transposed: U^T X^T = Z^T, a forward substitution in S = [U^T | Z^T]
+// with the tensor-core updates above.
+//
+// k_tinv_diag: D_R = diag(R) (mixed: diag(R_Y) D'), its reciprocals.
+// k_tinv_form: S[j][m] = U_mj = R_mj / D_m for m < j, S[j][rhs + i] = T^-1[i][perm j].
+// R: FP32 R_Y with D' (mixed path, R_mj = R_Y[m][j] D'_j), or complex128 with Dp null.
 template <typename T>
-cudaError_t launch_update(ftq_ctx* c, cx<T>* S, int ld, int jb, int nb, int r0, int r1, int c0, int c1) {
+__global__ void __launch_bounds__(256) k_tinv_diag(const cx<T>* __restrict__ R, const double2* __restrict__ Dp,
+                                                  double2* __restrict__ dinv, double2* __restrict__ DR,
+                                                  int* __restrict__ status, int M) {
+    const size_t w = blockIdx.x;
+    for (int j = threadIdx.x; j < M; j += 256) {
+        const cx<T> r = R[(w * M + j) * M + j];
+        double2 d = make_double2(r.x, r.y);
+        if (Dp) d = cmul(d, Dp[w * M + j]);
+        DR[w * M + j] = d;
+        if (!(abs2(d) > 0.0)) atomicOr(status, 1);
+        dinv[w * M + j] = cinv(d);
+    }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) k_tinv_form(const cx<T>* __restrict__ R, const double2* __restrict__ Dp,
+                                                  const double2* __restrict__ dinv, const int* __restrict__ perm,
+                                                  const double2* __restrict__ Tinv, double2* __restrict__ S, int M,
+                                                  int ld) {
+    __shared__ double2 tu[32][33];
+    __shared__ int pos[32];                                  // position of T^-1's column c0 + q
+    const int w = blockIdx.z, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32;    // rows and columns of R, or of T^-1
+    const size_t off = (size_t)w * M * M, so = (size_t)w * M;
+    double2* Sw = S + so * ld;
+    if (c0 + 31 > r0) {
+        for (int q = wid; q < 32; q += 8) {
+            const int m = r0 + q, j = c0 + lane;
+            if (m < j && j < M) {
+                const cx<T> r = R[off + (size_t)m * M + j];
+                double2 v = make_double2(r.x, r.y);
+                if (Dp) v = cmul(v, Dp[so + j]);
+                tu[q][lane] = cmul(v, dinv[so + m]);
+            }
+        }
+        __syncthreads();
+        for (int q = wid; q < 32; q += 8) {
+            const int j = c0 + q, m = r0 + lane;
+            if (m < j && j < M) Sw[(size_t)j * ld + m] = tu[lane][q];
+        }
+        __syncthreads();
+    }
+    for (int j = threadIdx.x; j < M; j += 256) {
+        const int c = perm[so + j] - c0;
+        if (c >= 0 && c < 32) pos[c] = j;
+    }
+    for (int q = wid; q < 32; q += 8) {
+        const int i = r0 + q, c = c0 + lane;
+        if (i < M && c < M) tu[q][lane] = Tinv[off + (size_t)i * M + c];
+    }
+    __syncthreads();
+    for (int q = wid; q < 32; q += 8) {
+        const int c = c0 + q, i = r0 + lane;
+        if (c < M && i < M) Sw[(size_t)pos[q] * ld + ld / 2 + i] = tu[lane][q];
+    }
+}
+
+// T^-1[i][j] = S[j][rhs + i].
+__global__ void __launch_bounds__(256) k_tinv_out(const double2* __restrict__ S, double2* __restrict__ Tinv,
+                                                 int* __restrict__ status, int M, int ld) {
+    __shared__ double2 t[32][33];
+    const int w = blockIdx.z, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
+    bool bad = false;
+    for (int q = wid; q < 32; q += 8) {
+        const int j = j0 + q, i = i0 + lane;
+        if (j < M && i < M) {
+            const double2 v = S[((size_t)w * M + j) * ld + ld / 2 + i];
+            t[q][lane] = v;
+            // finite: neither exponent field is all ones
+            bad = bad || ((__double2hiint(v.x) & 0x7ff00000) == 0x7ff00000) ||
+                  ((__double2hiint(v.y) & 0x7ff00000) == 0x7ff00000);
+        }
+    }
+    if (bad) atomicOr(status, 1);
+    __syncthreads();
+    for (int q = wid; q < 32; q += 8) {
+        const int i = i0 + q, j = j0 + lane;
+        if (i < M && j < M) Tinv[((size_t)w * M + i) * M + j] = t[lane][q];
+    }
+}
+
+template <typename T>
+cudaError_t launch_update(ftq_ctx* c, cx<T>* S, int ld, int jb, int nb, int r0, int r1, int c0, int c1,
+                          int kind = FTQ_K_GREEN) {
     using C = UpCfg<T>;
     UpArgs<T> a;
     a.S = S;
@@ -812,7 +942,7 @@ cudaError_t launch_update(ftq_ctx* c, cx<T>* S, int ld, int jb, int nb, int r0, 
     constexpr size_t sm = up_smem<T>();
     cudaError_t e = cudaFuncSetAttribute(k_lu_update<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    c->launches[FTQ_K_GREEN] += 1;
+    c->launches[kind] += 1;
     k_lu_update<T><<<std::min(sms, a.W * a.nrb * a.nct), NT_UP, sm, c->stream>>>(
         a, *reinterpret_cast<const CUtensorMap*>(c->lu_map[sizeof(T) == 8]));
     return cudaGetLastError();
@@ -879,6 +1009,48 @@ cudaError_t lu_make_maps(ftq_ctx* c) {
     bool ok = tc_map_3d(c->lu_map[1], c->work, 4 * ld, M, W, 16 * ld, 16 * ld * M, CROW / 4, CBOX);
     if (c->w32) ok = ok && tc_map_3d(c->lu_map[0], c->w32, 2 * ld, M, W, 8 * ld, 8 * ld * M, CROW / 4, CBOX);
     return ok ? cudaSuccess : cudaErrorNotSupported;
+}
+
+namespace {
+
+template <typename T>
+cudaError_t tinv_lu(ftq_ctx* c, const cx<T>* R, const double2* Dp, const int* perm, bool df) {
+    const int M = c->M, W = c->W, ld = lu_ld(M), rhs = ld / 2;
+    double2* S = c->work;
+    double2* dinv = scales_of<double>(c).inv;
+    const dim3 tiles((unsigned)((M + 31) / 32), (unsigned)((M + 31) / 32), (unsigned)W);
+    k_tinv_diag<T><<<W, 256, 0, c->stream>>>(R, Dp, dinv, c->DR, c->status, M);
+    k_tinv_form<T><<<tiles, 256, 0, c->stream>>>(R, Dp, dinv, perm, c->Tinv, S, M, ld);
+    c->launches[FTQ_K_TINV] += 2;
+    const int nblk = (M + 127) / 128, nt = ((M + nblk - 1) / nblk + 31) / 32 * 32;
+    const dim3 cols((unsigned)((M + nt - 1) / nt), (unsigned)W);
+    const size_t sm = sizeof(float4) * (32 * 32 + 32 * (size_t)nt);
+    cudaError_t e = cudaGetLastError();
+    if (df && e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_tinv_tri_df, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(sizeof(float4) * (32 * 32 + 32 * 128)));
+    for (int jb = 0; jb < M && e == cudaSuccess; jb += 32) {
+        const int nb = std::min(32, M - jb);
+        if (df) k_tinv_tri_df<<<cols, nt, sm, c->stream>>>(S, M, ld, jb, nb, rhs, rhs + M);
+        else k_lu_tri<double, 32, false, false><<<cols, nt, 0, c->stream>>>(S, scales_of<double>(c), M, ld, jb, nb, rhs, rhs + M);
+        c->launches[FTQ_K_TINV] += 1;
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = launch_update<double>(c, S, ld, jb, nb, jb + nb, M, rhs, rhs + M, FTQ_K_TINV);
+    }
+    if (e != cudaSuccess) return e;
+    k_tinv_out<<<tiles, 256, 0, c->stream>>>(S, c->Tinv, c->status, M, ld);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_tinv_lu32(ftq_ctx* c) {
+    LaunchScope ls(c, FTQ_K_TINV);
+    return tinv_lu<float>(c, c->w32, c->hh, c->perm, true);
+}
+
+cudaError_t launch_tinv_lu64(ftq_ctx* c, const double2* R, const int* perm) {
+    return tinv_lu<double>(c, R, nullptr, perm, false);
 }
 
 cudaError_t launch_green_lu64(ftq_ctx* c, const double2* Y, int k, bool update, bool physical) {

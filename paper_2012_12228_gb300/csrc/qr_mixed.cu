@@ -23,6 +23,7 @@
 #include <cmath>
 
 #include "complex_math.cuh"
+#include "df_math.cuh"
 #include "ftq_internal.h"
 #include "mixed_common.cuh"
 
@@ -418,40 +419,6 @@ __global__ void __launch_bounds__(288, 4) k_tinv64(const float2* __restrict__ A,
 //   shared memory and read at the same address by every thread; X column-major
 //   in double-FP32 in the scratch; T^-1 rows written back in FP64 through a
 //   shared tile.
-struct df2 { float h, l; };
-
-__device__ __forceinline__ df2 df_split(double v) {
-    df2 r;
-    r.h = (float)v;
-    r.l = (float)(v - (double)r.h);
-    return r;
-}
-
-// acc -= x * u  (x, u double-FP32; acc.l collects the rounding errors)
-__device__ __forceinline__ void df_msub(df2& acc, float xh, float xl, float uh, float ul) {
-    const float p = xh * uh;
-    float e = fmaf(xh, uh, -p);
-    e = fmaf(xh, ul, e);
-    e = fmaf(xl, uh, e);
-    const float t = acc.h - p;
-    const float bb = t - acc.h;
-    const float err = (acc.h - (t - bb)) + (-p - bb);
-    acc.h = t;
-    acc.l += err - e;
-}
-
-// acc += x * u
-__device__ __forceinline__ void df_madd(df2& acc, float xh, float xl, float uh, float ul) {
-    df_msub(acc, -xh, -xl, uh, ul);
-}
-
-__device__ __forceinline__ df2 df_norm(df2 a) {
-    df2 r;
-    r.h = a.h + a.l;
-    r.l = a.l - (r.h - a.h);
-    return r;
-}
-
 __global__ void __launch_bounds__(256) k_udt_prep(const float2* __restrict__ A, const double2* __restrict__ Dp,
                                                  float4* __restrict__ Udf, double2* __restrict__ DR,
                                                  int* __restrict__ status, int M) {
@@ -761,6 +728,12 @@ cudaError_t launch_tinv_df(ftq_ctx* c) {
     return cudaGetLastError();
 }
 
+// From this basis size on the T^-1 update runs as a forward substitution with
+// tensor-core updates (green_lu.cu).  Per stabilisation, k_tinv_df against it: M = 57, 640
+// walkers 0.35 / 0.40 ms, M = 123, 256 walkers 0.98 / 0.63, M = 257, 1024 walkers 23.0 /
+// 18.2, M = 515, 64 walkers 18.9 / 7.8.
+constexpr int TINV_LU_MIN_M = 100;
+
 cudaError_t launch_qr_prepiv(ftq_ctx* c) {
     const int M = c->M;
     Planes P;
@@ -775,7 +748,10 @@ cudaError_t launch_qr_prepiv(ftq_ctx* c) {
         e = launch_qr32(c, qr_panel_width(c));
         if (e != cudaSuccess) return e;
     }
-    if (c->opts.precision != FTQ_MIXED_F64UDT) {
+    if (c->opts.precision != FTQ_MIXED_F64UDT && M >= TINV_LU_MIN_M) {
+        e = launch_tinv_lu32(c);
+        if (e != cudaSuccess) return e;
+    } else if (c->opts.precision != FTQ_MIXED_F64UDT) {
         LaunchScope ls(c, FTQ_K_TINV);
         e = launch_tinv_df(c);
         if (e != cudaSuccess) return e;
