@@ -250,7 +250,7 @@ int ftq_status(ftq_ctx* ctx, int* status_host);
 
 /* Choose the mixed path's kernel for G(tau_k), k < n (no counterpart in the
  * paper, which computes G by one factorisation per slice): 0 by basis size
- * (tensor cores from M = 64 up), 1 the blocked LU with tensor-core updates,
+ * (tensor cores from M = 48 up), 1 the blocked LU with tensor-core updates,
  * 2 the CUDA-core blocked LU.  Both compute the same G, ln det and weights to
  * FP32 accuracy; ftq_autotune sets the faster one.  No effect for FP64
  * precision, FTQ_MIXED_SIMT (always the LU) or low rank.

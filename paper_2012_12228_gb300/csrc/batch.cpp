@@ -33,8 +33,14 @@ cudaError_t run_slices(ftq_ctx* b, int n, const double* const* fields) {
         const float* zin[8];
         float* out[8];
         int cur = 0;
+        // small bases run a slice's Horner steps in one launch, the others step by step together
+        for (int s = 0; s < ns; ++s)
+            if (ftq::chain_slice_fits(b->members[s])) {
+                cudaError_t e = ftq::chain_slice(b->members[s]);
+                if (e != cudaSuccess) return e;
+            }
         for (int s = 0; s < ns; ++s) zin[s] = b->members[s]->Ypl;
-        for (int j = p; j >= 1; --j) {
+        for (int j = p; j >= 1 && b->nitems > 0; --j) {
             for (int s = 0; s < ns; ++s) out[s] = b->members[s]->zpl[cur];
             cudaError_t e = ftq::tc_chain_step_batch(b, zin, out, j, p);
             if (e != cudaSuccess) return e;
@@ -43,6 +49,7 @@ cudaError_t run_slices(ftq_ctx* b, int n, const double* const* fields) {
         }
         for (int s = 0; s < ns; ++s) {
             ftq_ctx* m = b->members[s];
+            if (ftq::chain_slice_fits(m)) continue;          // done in place
             float* res = m->zpl[cur ^ 1];
             m->zpl[cur ^ 1] = m->Ypl;
             m->Ypl = res;

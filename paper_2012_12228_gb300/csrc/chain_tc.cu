@@ -750,6 +750,7 @@ cudaError_t tc_chain_step_batch(ftq_ctx* b, const float* const* zin, float* cons
         if (!fill_args(c, zin[s], out[s], j == p ? c->tab.h : nullptr, j == 1 ? c->tab.h : nullptr, 1.0f / j,
                        &tb.args[s], &tb.maps[s], &NT))
             return cudaErrorInvalidValue;
+        if (chain_slice_fits(c)) continue;      // not in the work list
         tb.nt_max = std::max(tb.nt_max, NT);
         tb.nslot_max = std::max(tb.nslot_max, c->nslot);
         tb.m_max = std::max(tb.m_max, c->M);
@@ -760,6 +761,7 @@ cudaError_t tc_chain_step_batch(ftq_ctx* b, const float* const* zin, float* cons
     cudaError_t e = launch_items(b, tb, b->items, b->nitems, b->stream);
     for (int s = 0; s < ns && e == cudaSuccess; ++s) {
         ftq_ctx* c = b->members[s];
+        if (chain_slice_fits(c)) continue;
         e = launch_border(c, zin[s], out[s], j == p ? c->tab.h : nullptr, j == 1 ? c->tab.h : nullptr, 1.0f / j);
     }
     return e;
@@ -822,6 +824,7 @@ cudaError_t tc_batch_items(ftq_ctx* b) {
     std::vector<int4> items;
     for (int s : order) {
         ftq_ctx* c = b->members[s];
+        if (chain_slice_fits(c)) continue;      // a slice in one launch of its own
         int R, NT;
         tc_plan(c->M, c->nct, &R, &NT);
         for (int w = 0; w < c->W; ++w)
@@ -830,9 +833,10 @@ cudaError_t tc_batch_items(ftq_ctx* b) {
     }
     if (b->items) cudaFree(b->items);
     b->items = nullptr;
+    b->nitems = (int)items.size();
+    if (items.empty()) return cudaSuccess;
     cudaError_t e = cudaMalloc(&b->items, sizeof(int4) * items.size());
     if (e != cudaSuccess) return e;
-    b->nitems = (int)items.size();
     return cudaMemcpy(b->items, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice);
 }
 

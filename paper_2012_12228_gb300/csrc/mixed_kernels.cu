@@ -384,6 +384,7 @@ cudaError_t mixed_init(ftq_ctx* c) {
 }
 
 cudaError_t mixed_chain(ftq_ctx* c) {
+    if (chain_slice_fits(c)) return chain_slice(c);
     const int M = c->M, p = c->opts.exp_order;
     const bool tensor = c->opts.precision == FTQ_MIXED || c->opts.precision == FTQ_MIXED_F64UDT;
     const int tiles = (M + ST - 1) / ST;
@@ -496,11 +497,10 @@ cudaError_t mixed_green(ftq_ctx* c, int k) {
 // per walker.  Measured on a GB300, ms per slice (tensor cores / CUDA cores):
 // M = 7, 64 walkers 0.059 / 0.035; M = 33, 300 walkers 0.130 / 0.114; M = 57, 640
 // walkers 0.240 / 0.437; M = 123, 256 walkers 0.43 / 0.71; M = 257, 1024 walkers
-// 7.5 / 9.4; M = 257, 64 walkers 0.88 / 2.5; M = 515, 64 walkers 3.4 / 17.0.  Without a
-// measurement the tensor cores take over above M = 57, where FP32 rounding of either
-// kernel leaves the drift of the mixed chain least room; ftq_autotune times both on
-// the context's own workload.
-constexpr int GREEN_TC_MIN_M = 64;
+// 7.5 / 9.4; M = 257, 64 walkers 0.88 / 2.5; M = 515, 64 walkers 3.4 / 17.0.  The line
+// lies between the closed shells 33 and 57; ftq_autotune times both on the
+// context's own workload.
+constexpr int GREEN_TC_MIN_M = 48;
 
 bool green_uses_tc(const ftq_ctx* c) {
     if (c->opts.precision == FTQ_MIXED_SIMT) return false;
