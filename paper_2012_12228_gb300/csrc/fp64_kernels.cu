@@ -131,7 +131,8 @@ __global__ void k_qrcp(const double2* __restrict__ Yin, double2* __restrict__ Qo
                        double2* __restrict__ work, double2* __restrict__ work2,
                        double2* __restrict__ DR, double2* __restrict__ Tinv,
                        double2* __restrict__ hh, double* __restrict__ htau,
-                       double* __restrict__ ws, int* __restrict__ status, int* __restrict__ perm_out, int M) {
+                       double* __restrict__ ws, int* __restrict__ status, int* __restrict__ perm_out, int M,
+                       int in_smem) {
     extern __shared__ unsigned char smem_raw[];
     double* cn = reinterpret_cast<double*>(smem_raw);          // column norms [M]
     int* perm = reinterpret_cast<int*>(cn + M);                 // [M]
@@ -140,9 +141,11 @@ __global__ void k_qrcp(const double2* __restrict__ Yin, double2* __restrict__ Qo
     __shared__ int nswap;
     const int w = blockIdx.x;
     const long off = (long)w * M * M;
-    double2* C = work + off;
-    double2* Q = Qout + off;
-    double2* XT = work2 + off;
+    // small bases: the three matrices in shared memory (fact_smem)
+    double2* mats = reinterpret_cast<double2*>(smem_raw + ((12 * (size_t)M + 15) & ~(size_t)15));
+    double2* C = in_smem ? mats : work + off;
+    double2* Q = in_smem ? mats + M * M : Qout + off;
+    double2* XT = in_smem ? mats + 2 * M * M : work2 + off;
     double2* Ti = Tinv + off;
     const double2* Yw = Yin + off;
     double2* u0 = hh + (long)w * M;
@@ -157,13 +160,19 @@ __global__ void k_qrcp(const double2* __restrict__ Yin, double2* __restrict__ Qo
     if (threadIdx.x == 0) nswap = 0;
     __syncthreads();
 
+    // norms of the columns; after that every reflector's update leaves those of the
+    // rows below it, so that no pass over the matrix is spent on them
+    for (int c = threadIdx.x; c < M; c += nt) {
+        double s = 0.0;
+        for (int r = 0; r < M; ++r) s += abs2(C[(long)r * M + c]);
+        cn[c] = s;
+    }
+    __syncthreads();
     for (int j = 0; j < M; ++j) {
         double best = -1.0;
         int bidx = M;
         for (int c = j + threadIdx.x; c < M; c += nt) {
-            double s = 0.0;
-            for (int r = j; r < M; ++r) s += abs2(C[(long)r * M + c]);
-            cn[c] = s;
+            const double s = cn[c];
             if (s > best) { best = s; bidx = c; }
         }
         int pc = block_argmax(best, bidx, shv, shi);
@@ -203,7 +212,13 @@ __global__ void k_qrcp(const double2* __restrict__ Yin, double2* __restrict__ Qo
             for (int r = j + 1; r < M; ++r) s = cfma(conj(C[(long)r * M + j]), C[(long)r * M + c], s);
             s = s * tj;
             C[(long)j * M + c] = cfms(uj, s, C[(long)j * M + c]);
-            for (int r = j + 1; r < M; ++r) C[(long)r * M + c] = cfms(C[(long)r * M + j], s, C[(long)r * M + c]);
+            double left = 0.0;
+            for (int r = j + 1; r < M; ++r) {
+                const double2 v = cfms(C[(long)r * M + j], s, C[(long)r * M + c]);
+                C[(long)r * M + c] = v;
+                left += abs2(v);
+            }
+            cn[c] = left;
         }
         __syncthreads();
     }
@@ -225,6 +240,8 @@ __global__ void k_qrcp(const double2* __restrict__ Yin, double2* __restrict__ Qo
         }
         __syncthreads();
     }
+    if (in_smem)
+        for (int e = threadIdx.x; e < M * M; e += nt) Qout[off + e] = Q[e];
     if (perm_out) {                          // T^-1 is updated from R by the kernels of green_lu.cu
         for (int j = threadIdx.x; j < M; j += nt) perm_out[(long)w * M + j] = perm[j];
         if (threadIdx.x == 0) {
@@ -266,7 +283,7 @@ __global__ void k_green(const double2* __restrict__ Y, const double2* __restrict
                         double2* __restrict__ work2, double2* __restrict__ G,
                         const double* __restrict__ eps, double* __restrict__ ws,
                         int* __restrict__ status, int M, double lscale, double mu_T,
-                        int constraint, int update, int with_gauss, double kdt) {
+                        int constraint, int update, int with_gauss, double kdt, int in_smem) {
     extern __shared__ unsigned char smem_raw[];
     double2* drs = reinterpret_cast<double2*>(smem_raw);     // [M]
     double2* invU = drs + M;                                 // [M]
@@ -281,8 +298,10 @@ __global__ void k_green(const double2* __restrict__ Y, const double2* __restrict
     const int w = blockIdx.x;
     const long off = (long)w * M * M;
     const int nt = blockDim.x;
-    double2* A = work + off;
-    double2* XT = work2 + off;
+    // small bases: both matrices in shared memory (fact_smem)
+    double2* mats = reinterpret_cast<double2*>(smem_raw + ((60 * (size_t)M + 15) & ~(size_t)15));
+    double2* A = in_smem ? mats : work + off;
+    double2* XT = in_smem ? mats + M * M : work2 + off;
     const double2* Yw = Y + off;
     const double2* Tw = Tinv + off;
     double2* Gw = G + off;
@@ -378,6 +397,16 @@ __global__ void k_green(const double2* __restrict__ Y, const double2* __restrict
     }
 }
 
+// The one-block factorisations of bases below lu64_supported's keep their matrices in
+// shared memory (two for G, three for the QRCP; at most 106 KB at M = 47).  Per launch
+// at M = 33, 300 walkers: G 378 -> 350 us, QRCP 670 -> 618 us; what remains is the FP64
+// pipe with 33 of 64 lanes in use.
+constexpr int SMEM_M = 47;
+
+size_t fact_smem(int M, size_t vectors, int matrices) {
+    return M <= SMEM_M ? ((vectors + 15) & ~(size_t)15) + sizeof(double2) * matrices * (size_t)M * M : vectors;
+}
+
 int fact_threads(int M) {
     int t = ((M + 31) / 32) * 32;
     return t > 1024 ? 1024 : (t < 32 ? 32 : t);
@@ -427,13 +456,17 @@ cudaError_t launch_chain(ftq_ctx* c) {
 
 cudaError_t launch_qrcp64(ftq_ctx* c, const double2* Yin, double2* Qout) {
     const int M = c->M;
-    size_t sm = sizeof(double) * M + sizeof(int) * M;
+    const size_t sm = fact_smem(M, (sizeof(double) + sizeof(int)) * M, 3);
     int nt = fact_threads(M);
+    if (sm > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(k_qrcp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (e != cudaSuccess) return e;
+    }
     const bool lu = lu64_supported(M);
     double2* R = lu ? c->zbuf[1] : c->work;      // S of the T^-1 update takes the work buffer
     LaunchScope ls(c, FTQ_K_QRCP);
     k_qrcp<<<c->W, nt, sm, c->stream>>>(Yin, Qout, R, c->work2, c->DR, c->Tinv, c->hh, c->htau,
-                                       c->wstate, c->status, lu ? c->perm : nullptr, M);
+                                       c->wstate, c->status, lu ? c->perm : nullptr, M, M <= SMEM_M ? 1 : 0);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && lu) e = launch_tinv_lu64(c, R, c->perm);
     return e;
@@ -458,14 +491,14 @@ cudaError_t launch_green64(ftq_ctx* c, const double2* Y, int k, bool update, boo
     const int M = c->M;
     if (c->opts.low_rank_threshold > 0.0) return launch_green_lr(c, Y, k, update, physical);
     if (lu64_supported(M)) return launch_green_lu64(c, Y, k, update, physical);
-    size_t sm = (2 * sizeof(double2) + 3 * sizeof(double) + sizeof(int)) * M;
+    const size_t sm = fact_smem(M, (2 * sizeof(double2) + 3 * sizeof(double) + sizeof(int)) * M, 2);
     int nt = fact_threads(M);
     const double lscale = physical ? 0.0 : left_scale(c, k);
     if (sm > 48 * 1024) cudaFuncSetAttribute(k_green, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     LaunchScope ls(c, FTQ_K_GREEN);
     k_green<<<c->W, nt, sm, c->stream>>>(Y, c->Tinv, c->DR, c->work, c->work2, c->G, c->tab.eps, c->wstate,
                                         c->status, M, lscale, c->sys.mu_T, c->opts.constraint, update ? 1 : 0,
-                                        physical ? 0 : 1, (double)k * c->sys.dtau);
+                                        physical ? 0 : 1, (double)k * c->sys.dtau, M <= SMEM_M ? 1 : 0);
     return cudaGetLastError();
 }
 

@@ -54,13 +54,19 @@ __device__ int qrcp_panel(double2* A, int ld, int rows, int cols, int kmax, int*
     for (int c = threadIdx.x; c < cols; c += nt) perm[c] = c;
     if (threadIdx.x == 0) nswap = 0;
     __syncthreads();
+    // norms of the columns; after that every reflector's update leaves those of the
+    // rows below it
+    for (int c = threadIdx.x; c < cols; c += nt) {
+        double s = 0.0;
+        for (int r = 0; r < rows; ++r) s += abs2(A[(long)r * ld + c]);
+        cn[c] = s;
+    }
+    __syncthreads();
     for (int j = 0; j < kmax; ++j) {
         double best = -1.0;
         int bidx = cols;
         for (int c = j + threadIdx.x; c < cols; c += nt) {
-            double s = 0.0;
-            for (int r = j; r < rows; ++r) s += abs2(A[(long)r * ld + c]);
-            cn[c] = s;
+            const double s = cn[c];
             if (s > best) { best = s; bidx = c; }
         }
         int pc = block_argmax(best, bidx, shv, shi);
@@ -90,7 +96,13 @@ __device__ int qrcp_panel(double2* A, int ld, int rows, int cols, int kmax, int*
             for (int r = j + 1; r < rows; ++r) s = cfma(conj(A[(long)r * ld + j]), A[(long)r * ld + c], s);
             s = s * tj;
             A[(long)j * ld + c] = cfms(uj, s, A[(long)j * ld + c]);
-            for (int r = j + 1; r < rows; ++r) A[(long)r * ld + c] = cfms(A[(long)r * ld + j], s, A[(long)r * ld + c]);
+            double left = 0.0;
+            for (int r = j + 1; r < rows; ++r) {
+                const double2 v = cfms(A[(long)r * ld + j], s, A[(long)r * ld + c]);
+                A[(long)r * ld + c] = v;
+                left += abs2(v);
+            }
+            cn[c] = left;
         }
         __syncthreads();
     }
