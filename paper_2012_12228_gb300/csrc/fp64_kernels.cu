@@ -2,12 +2,14 @@
 // QRCP stabilisation, and the two-sided stable Green's function with ln det and
 // the phaseless weight (the chain is in chain_oz.cu, the estimators in
 // estimators.cu).  One walker per thread block for the factorisations.
+#include <algorithm>
 #include <cmath>
 
 #include "block_reduce.cuh"
 #include "complex_math.cuh"
 #include "ftq_internal.h"
 #include "green_tail.cuh"
+#include "reflect.cuh"
 
 namespace ftq {
 namespace {
@@ -205,21 +207,7 @@ __global__ void k_qrcp(const double2* __restrict__ Yin, double2* __restrict__ Qo
             if (!(sig > 0.0)) atomicOr(status, 1);
         }
         __syncthreads();
-        const double2 uj = u0[j];
-        const double tj = tau[j];
-        for (int c = j + 1 + threadIdx.x; c < M; c += nt) {
-            double2 s = cmul(conj(uj), C[(long)j * M + c]);
-            for (int r = j + 1; r < M; ++r) s = cfma(conj(C[(long)r * M + j]), C[(long)r * M + c], s);
-            s = s * tj;
-            C[(long)j * M + c] = cfms(uj, s, C[(long)j * M + c]);
-            double left = 0.0;
-            for (int r = j + 1; r < M; ++r) {
-                const double2 v = cfms(C[(long)r * M + j], s, C[(long)r * M + c]);
-                C[(long)r * M + c] = v;
-                left += abs2(v);
-            }
-            cn[c] = left;
-        }
+        reflect_columns<true>(C, M, j, C, M, M, j + 1, M, u0[j], tau[j], cn);
         __syncthreads();
     }
     // Q = H_0 H_1 ... H_{M-1} by backward accumulation
@@ -229,15 +217,7 @@ __global__ void k_qrcp(const double2* __restrict__ Yin, double2* __restrict__ Qo
     }
     __syncthreads();
     for (int j = M - 1; j >= 0; --j) {
-        const double2 uj = u0[j];
-        const double tj = tau[j];
-        for (int c = j + threadIdx.x; c < M; c += nt) {
-            double2 s = cmul(conj(uj), Q[(long)j * M + c]);
-            for (int r = j + 1; r < M; ++r) s = cfma(conj(C[(long)r * M + j]), Q[(long)r * M + c], s);
-            s = s * tj;
-            Q[(long)j * M + c] = cfms(uj, s, Q[(long)j * M + c]);
-            for (int r = j + 1; r < M; ++r) Q[(long)r * M + c] = cfms(C[(long)r * M + j], s, Q[(long)r * M + c]);
-        }
+        reflect_columns<false>(C, M, j, Q, M, M, j, M, u0[j], tau[j], nullptr);
         __syncthreads();
     }
     if (in_smem)
@@ -457,7 +437,7 @@ cudaError_t launch_chain(ftq_ctx* c) {
 cudaError_t launch_qrcp64(ftq_ctx* c, const double2* Yin, double2* Qout) {
     const int M = c->M;
     const size_t sm = fact_smem(M, (sizeof(double) + sizeof(int)) * M, 3);
-    int nt = fact_threads(M);
+    const int nt = std::min(1024, 2 * fact_threads(M));      // two lanes per column
     if (sm > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k_qrcp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;

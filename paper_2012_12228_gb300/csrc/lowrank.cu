@@ -21,6 +21,7 @@
 #include "block_reduce.cuh"
 #include "complex_math.cuh"
 #include "ftq_internal.h"
+#include "reflect.cuh"
 
 namespace ftq {
 namespace {
@@ -89,21 +90,7 @@ __device__ int qrcp_panel(double2* A, int ld, int rows, int cols, int kmax, int*
         __syncthreads();
         if (threadIdx.x == 0) reflector(A, ld, j, cn[j], u0, tau, status);
         __syncthreads();
-        const double2 uj = u0[j];
-        const double tj = tau[j];
-        for (int c = j + 1 + threadIdx.x; c < cols; c += nt) {
-            double2 s = cmul(conj(uj), A[(long)j * ld + c]);
-            for (int r = j + 1; r < rows; ++r) s = cfma(conj(A[(long)r * ld + j]), A[(long)r * ld + c], s);
-            s = s * tj;
-            A[(long)j * ld + c] = cfms(uj, s, A[(long)j * ld + c]);
-            double left = 0.0;
-            for (int r = j + 1; r < rows; ++r) {
-                const double2 v = cfms(A[(long)r * ld + j], s, A[(long)r * ld + c]);
-                A[(long)r * ld + c] = v;
-                left += abs2(v);
-            }
-            cn[c] = left;
-        }
+        reflect_columns<true>(A, ld, j, A, ld, rows, j + 1, cols, u0[j], tau[j], cn);
         __syncthreads();
     }
     const int par = nswap;
@@ -123,15 +110,7 @@ __device__ void form_q(const double2* A, int lda, double2* Q, int ldq, int rows,
     }
     __syncthreads();
     for (int j = kmax - 1; j >= 0; --j) {
-        const double2 uj = u0[j];
-        const double tj = tau[j];
-        for (int c = j + threadIdx.x; c < kmax; c += nt) {
-            double2 s = cmul(conj(uj), Q[(long)j * ldq + c]);
-            for (int r = j + 1; r < rows; ++r) s = cfma(conj(A[(long)r * lda + j]), Q[(long)r * ldq + c], s);
-            s = s * tj;
-            Q[(long)j * ldq + c] = cfms(uj, s, Q[(long)j * ldq + c]);
-            for (int r = j + 1; r < rows; ++r) Q[(long)r * ldq + c] = cfms(A[(long)r * lda + j], s, Q[(long)r * ldq + c]);
-        }
+        reflect_columns<false>(A, lda, j, Q, ldq, rows, j, kmax, u0[j], tau[j], nullptr);
         __syncthreads();
     }
 }
@@ -140,7 +119,7 @@ __device__ void form_q(const double2* A, int lda, double2* Q, int ldq, int rows,
 // QRCP of C = Y[:, :m] diag(D) (M x m); D <- diag R over the kept prefix
 // |R_jj| >= thr (at least one), T <- (D^-1 R)(Pi T) restricted to the kept
 // rows, Q -> Qout (first m' columns), rank m' -> ws[12].
-constexpr int LR_THREADS = 512;
+constexpr int LR_THREADS = 576;
 
 __global__ void __launch_bounds__(LR_THREADS) k_qrcp_lr(const double2* __restrict__ Yin, double2* __restrict__ Qout, double2* __restrict__ work,
                           double2* __restrict__ work2, double2* __restrict__ DR, double2* __restrict__ Tm,
@@ -397,7 +376,7 @@ __global__ void __launch_bounds__(LR_THREADS) k_green_lr(const double2* __restri
 }
 
 int lr_threads(int M) {
-    int t = ((M + 31) / 32) * 32;
+    int t = 2 * (((M + 31) / 32) * 32);          // two lanes per column of a reflector's update
     return t > LR_THREADS ? LR_THREADS : (t < 32 ? 32 : t);
 }
 
