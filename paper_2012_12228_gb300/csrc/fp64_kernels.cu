@@ -129,7 +129,7 @@ __global__ void k_force_bias(const GT* __restrict__ G, const double* __restrict_
 // Reflector H = I - tau u u^H with u = x - beta e_1, beta = -e^{i arg x_0}|x|,
 // so H x = beta e_1 and R_jj = beta.  Outputs: Q (next chain start), D_R =
 // diag R, T^-1 <- T^-1 Pi^T (D^-1 R)^-1, parity of Pi.
-__global__ void k_qrcp(const double2* __restrict__ Yin, double2* __restrict__ Qout,
+__global__ void __launch_bounds__(1024) k_qrcp(const double2* __restrict__ Yin, double2* __restrict__ Qout,
                        double2* __restrict__ work, double2* __restrict__ work2,
                        double2* __restrict__ DR, double2* __restrict__ Tinv,
                        double2* __restrict__ hh, double* __restrict__ htau,
@@ -258,7 +258,22 @@ __global__ void k_qrcp(const double2* __restrict__ Yin, double2* __restrict__ Qo
 //   ln det(I + A) = -sum ln D_Lb - sum ln D_Rb + ln det Mt + ln det T,
 // then ln S_k = 2 (ln det_k - ln det_{k-1}) and the weight (Eqs. import,
 // phimport, theta).
-__global__ void k_green(const double2* __restrict__ Y, const double2* __restrict__ Tinv,
+//
+// L lanes share a column of the LU's updates and a row of the solves: four for the
+// small bases, where a lane per row left half of a block's lanes idle and the
+// sums' latency exposed.
+template <int L>
+__device__ __forceinline__ double2 lane_sum(double2 s) {
+#pragma unroll
+    for (int o = 1; o < L; o <<= 1) {
+        s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+        s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+    }
+    return s;
+}
+
+template <int L>
+__global__ void __launch_bounds__(1024) k_green(const double2* __restrict__ Y, const double2* __restrict__ Tinv,
                         const double2* __restrict__ DR, double2* __restrict__ work,
                         double2* __restrict__ work2, double2* __restrict__ G,
                         const double* __restrict__ eps, double* __restrict__ ws,
@@ -278,6 +293,7 @@ __global__ void k_green(const double2* __restrict__ Y, const double2* __restrict
     const int w = blockIdx.x;
     const long off = (long)w * M * M;
     const int nt = blockDim.x;
+    const int q = threadIdx.x % L;
     // small bases: both matrices in shared memory (fact_smem)
     double2* mats = reinterpret_cast<double2*>(smem_raw + ((60 * (size_t)M + 15) & ~(size_t)15));
     double2* A = in_smem ? mats : work + off;
@@ -336,9 +352,9 @@ __global__ void k_green(const double2* __restrict__ Y, const double2* __restrict
         for (int i = j + 1 + threadIdx.x; i < M; i += nt) A[(long)i * M + j] = cmul(A[(long)i * M + j], ip);
         if (threadIdx.x == 0) invU[j] = ip;
         __syncthreads();
-        for (int c = j + 1 + threadIdx.x; c < M; c += nt) {
+        for (int c = j + 1 + (int)threadIdx.x / L; c < M; c += nt / L) {
             const double2 u = A[(long)j * M + c];
-            for (int i = j + 1; i < M; ++i) A[(long)i * M + c] = cfms(A[(long)i * M + j], u, A[(long)i * M + c]);
+            for (int i = j + 1 + q; i < M; i += L) A[(long)i * M + c] = cfms(A[(long)i * M + j], u, A[(long)i * M + c]);
         }
         __syncthreads();
     }
@@ -349,18 +365,31 @@ __global__ void k_green(const double2* __restrict__ Y, const double2* __restrict
     lsum = block_sum(lsum, shv);
     // X = (Y D_Rs) U^-1 L^-1 solved row by row (XT column-major), then
     // G[i][perm[m]] = delta - X[i][m] dls[perm[m]].
-    for (int i = threadIdx.x; i < M; i += nt) {
+    // L lanes share a row and its sums (the same trips for every lane of a warp)
+    for (int ib = 0; ib < M; ib += nt / L) {
+        const int i = ib + (int)threadIdx.x / L;
+        const bool on = i < M;
         for (int j = 0; j < M; ++j) {
-            double2 s = cmul(Yw[(long)i * M + j], drs[j]);
-            for (int m = 0; m < j; ++m) s = cfms(XT[(long)m * M + i], A[(long)m * M + j], s);
-            XT[(long)j * M + i] = cmul(s, invU[j]);
+            double2 s = make_double2(0.0, 0.0);
+            if (on) {
+                if (q == 0) s = cmul(Yw[(long)i * M + j], drs[j]);
+                for (int m = q; m < j; m += L) s = cfms(XT[(long)m * M + i], A[(long)m * M + j], s);
+            }
+            s = lane_sum<L>(s);
+            if (on && q == 0) XT[(long)j * M + i] = cmul(s, invU[j]);
+            __syncwarp();
         }
         for (int j = M - 2; j >= 0; --j) {
-            double2 s = XT[(long)j * M + i];
-            for (int m = j + 1; m < M; ++m) s = cfms(XT[(long)m * M + i], A[(long)m * M + j], s);
-            XT[(long)j * M + i] = s;
+            double2 s = make_double2(0.0, 0.0);
+            if (on) {
+                if (q == 0) s = XT[(long)j * M + i];
+                for (int m = j + 1 + q; m < M; m += L) s = cfms(XT[(long)m * M + i], A[(long)m * M + j], s);
+            }
+            s = lane_sum<L>(s);
+            if (on && q == 0) XT[(long)j * M + i] = s;
+            __syncwarp();
         }
-        for (int m = 0; m < M; ++m) {
+        for (int m = q; m < M && on; m += L) {
             int c = perm[m];
             double2 g = XT[(long)m * M + i] * (-dls[c]);
             if (c == i) g.x += 1.0;
@@ -379,8 +408,8 @@ __global__ void k_green(const double2* __restrict__ Y, const double2* __restrict
 
 // The one-block factorisations of bases below lu64_supported's keep their matrices in
 // shared memory (two for G, three for the QRCP; at most 106 KB at M = 47).  Per launch
-// at M = 33, 300 walkers: G 378 -> 350 us, QRCP 670 -> 618 us; what remains is the FP64
-// pipe with 33 of 64 lanes in use.
+// at M = 33, 300 walkers: G 378 -> 350 us (314 with four lanes per row), QRCP 670 -> 618 us
+// (468 with two lanes per column).
 constexpr int SMEM_M = 47;
 
 size_t fact_smem(int M, size_t vectors, int matrices) {
@@ -472,13 +501,15 @@ cudaError_t launch_green64(ftq_ctx* c, const double2* Y, int k, bool update, boo
     if (c->opts.low_rank_threshold > 0.0) return launch_green_lr(c, Y, k, update, physical);
     if (lu64_supported(M)) return launch_green_lu64(c, Y, k, update, physical);
     const size_t sm = fact_smem(M, (2 * sizeof(double2) + 3 * sizeof(double) + sizeof(int)) * M, 2);
-    int nt = fact_threads(M);
     const double lscale = physical ? 0.0 : left_scale(c, k);
-    if (sm > 48 * 1024) cudaFuncSetAttribute(k_green, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const bool small = M <= SMEM_M;
+    auto kernel = small ? k_green<4> : k_green<1>;
+    const int nt = small ? (4 * M + 31) / 32 * 32 : fact_threads(M);
+    if (sm > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     LaunchScope ls(c, FTQ_K_GREEN);
-    k_green<<<c->W, nt, sm, c->stream>>>(Y, c->Tinv, c->DR, c->work, c->work2, c->G, c->tab.eps, c->wstate,
-                                        c->status, M, lscale, c->sys.mu_T, c->opts.constraint, update ? 1 : 0,
-                                        physical ? 0 : 1, (double)k * c->sys.dtau, M <= SMEM_M ? 1 : 0);
+    kernel<<<c->W, nt, sm, c->stream>>>(Y, c->Tinv, c->DR, c->work, c->work2, c->G, c->tab.eps, c->wstate,
+                                       c->status, M, lscale, c->sys.mu_T, c->opts.constraint, update ? 1 : 0,
+                                       physical ? 0 : 1, (double)k * c->sys.dtau, small ? 1 : 0);
     return cudaGetLastError();
 }
 
