@@ -182,7 +182,6 @@ def set_device_peaks(torch, dev):
 TRAFFIC_PER_WALKER = {     # (bytes per walker, summary file, walkers in the capture)
     ("mixed", "green"): ((15.221e9 + 4.772e9) / 608, "profiles/green32b_ueg_n66_m257_w608.md", 608),
     ("mixed", "chain"): ((0.43736e9 + 0.22356e9) / 256, "profiles/chain_tc_ueg_n66_m257_w256.md", 256),
-    ("fp64", "chain"): (0.3867e9 / 128, "profiles/chain_fp64_ueg_n66_m257_w128.md", 128),
 }
 
 
@@ -201,14 +200,20 @@ def kernel_model(kind, M, W, precision, green_tc=False):
     tf32 = ("tensor", bf16 * 1.1 / 2.25,
             f"tf32 dense = measured bf16 {bf16:.1f} TFLOP/s x 1.1/2.25 (MEASURED_PEAKS.json)"
             if "bf16_tflops" in PEAKS else "tf32 dense = fallback bf16 1900 TFLOP/s x 1.1/2.25")
+    # complex128 products as 36 products of bf16 digits (bases above 19 in the chain, above 47 elsewhere)
+    digits = ("tensor", bf16, f"bf16 dense = {bf16:.1f} TFLOP/s (MEASURED_PEAKS.json), 36 digit products per FP64 one")
     if kind == "chain":          # one Horner step: V (M x M) times Z (M x M), per walker
         if precision == "mixed":
             return (3 * 8.0 * M ** 3 * W,) + tf32
+        if precision == "fp64" and M > 19:
+            return (36 * 8.0 * M ** 3 * W,) + digits
         return (8.0 * M ** 3 * W,) + (fp64 if precision == "fp64" else fp32)
     if kind == "green":
         if green_tc:             # elimination of [Mt^T | B^T] on the tensor cores, counted as 1.5 M^3 complex
                                  # MACs at tf32 cost (six bf16 products each; the blocked LU needs 4/3 M^3)
             return (3 * 12.0 * M ** 3 * W,) + tf32
+        if precision == "fp64" and 48 <= M <= 640:
+            return (36 * (8.0 / 3.0 + 8.0) * M ** 3 * W,) + digits
         # LU (8/3 M^3) + two triangular solves with M right-hand sides (8 M^3)
         return ((8.0 / 3.0 + 8.0) * M ** 3 * W,) + (fp64 if precision == "fp64" else fp32)
     if kind == "qrcp":
@@ -216,6 +221,8 @@ def kernel_model(kind, M, W, precision, green_tc=False):
             return ((16.0 / 3.0 + 16.0 / 3.0 + 4.0) * M ** 3 * W,) + fp64
         return ((16.0 / 3.0) * M ** 3 * W,) + fp32          # FP32 Householder of Y Pi (Q: bridge class)
     if kind == "tinv":           # T^-1 <- T^-1 Pi U^-1: a triangular solve with M right-hand sides
+        if M >= 100:
+            return (36 * 4.0 * M ** 3 * W,) + digits
         return (4.0 * M ** 3 * W,) + fp64
     return None
 
@@ -332,7 +339,10 @@ def measure_path(ftq, torch, dev, precision, W, steps, warmup, world, rank, barr
     prop.estimators(per_walker=False)
     after = prop.profile_read()
     prop.profile(False)
-    prof = {k: {"ms": after[k][0], "n_timed": after[k][1] - before[k][1]} for k in after}
+    # operations of the block, not launches: an evaluation of G is many launches
+    ops = {"chain": p_order * stab, "green": stab, "qrcp": 1, "tinv": 1}
+    prof = {k: {"ms": after[k][0], "n_timed": ops.get(k, after[k][1] - before[k][1]) if after[k][0] > 0 else 0}
+            for k in after}
     out["kernel_ms_per_step"] = {k: v["ms"] for k, v in prof.items() if v["ms"] > 0}
     out["roofline"] = roofline(prof, M, W, precision, green_tc=prop.query("GREEN_KERNEL") == 1)
     out["device_status"] = prop.status()
@@ -463,7 +473,7 @@ def ragged_roofline(b, fl, stab, ctxs):
     model = None
     for sd, m in zip(RAGGED, b.members):
         per_block = {"chain": 6 * stab, "green": stab, "qrcp": 1, "tinv": 1}.get(dom, 0)
-        mm = kernel_model(dom, m.M, m.W, "mixed")
+        mm = kernel_model(dom, m.M, m.W, "mixed", m.query("GREEN_KERNEL") == 1)
         if mm is None or per_block == 0:
             model = None
             break

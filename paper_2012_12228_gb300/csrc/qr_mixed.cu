@@ -16,7 +16,9 @@
 //       D', and A = Y Pi (FP32, row-major).
 //   k_qr32 (one block per walker): blocked Householder QR of A in FP32
 //       (compact WY panels of NB columns); R_Y in A, reflectors and tau out.
-//   k_tinv64 (FP64, one block per walker): D_R, U and T^-1 <- T^-1 Pi U^-1.
+//   D_R, U and T^-1 <- T^-1 Pi U^-1: the substitution kernels of green_lu.cu for large
+//       bases, k_udt_prep and k_tinv_df (double-FP32) for small ones, k_tinv64 (FP64, one
+//       block per walker) with FTQ_MIXED_F64UDT.
 //   k_form_q32 (FP32, one block per walker and 32- or 16-column panel): Q = H_0 ...
 //       H_{M-1} applied to the identity panel in shared memory, written into
 //       the chain planes as the new Y.
