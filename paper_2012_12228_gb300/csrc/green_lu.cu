@@ -999,8 +999,8 @@ size_t lu_scal_doubles(int M, int W) { return (size_t)W * (7 * (size_t)M + 1); }
 size_t lu_ints(int W) { return (size_t)W * (1 + 2 * LU_NB_MAX); }
 
 // Smaller bases keep the one-block k_green: at M = 33, 300 walkers a slice takes
-// 0.38 ms there and 0.57 ms here (launches and half-empty tiles), at M = 57, 256
-// walkers 1.20 against 0.75 ms.  Above, a panel row no longer fits a thread.
+// 0.31 ms there and 0.57 ms here (launches and half-empty tiles), at M = 57, 256
+// walkers 1.20 against 0.72 ms.  Above, a panel row no longer fits a thread.
 bool lu64_supported(int M) { return M >= 48 && M <= 640; }
 
 // Maps of S over the buffers it lives in: [W][M][ld], a row as floats.

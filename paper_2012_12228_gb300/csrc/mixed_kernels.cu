@@ -495,9 +495,9 @@ cudaError_t mixed_green(ftq_ctx* c, int k) {
 // Which Green kernel the mixed path runs for slices k < n: the blocked LU whose
 // updates run on the tensor cores (green_lu.cu), or the CUDA-core LU with one block
 // per walker.  Measured on a GB300, ms per slice (tensor cores / CUDA cores):
-// M = 7, 64 walkers 0.059 / 0.035; M = 33, 300 walkers 0.130 / 0.114; M = 57, 640
-// walkers 0.240 / 0.437; M = 123, 256 walkers 0.43 / 0.71; M = 257, 1024 walkers
-// 7.5 / 9.4; M = 257, 64 walkers 0.88 / 2.5; M = 515, 64 walkers 3.4 / 17.0.  The line
+// M = 7, 64 walkers 0.061 / 0.035; M = 33, 300 walkers 0.127 / 0.113; M = 57, 640
+// walkers 0.235 / 0.438; M = 123, 256 walkers 0.42 / 0.71; M = 257, 1024 walkers
+// 7.1 / 9.4; M = 257, 64 walkers 0.84 / 2.5; M = 515, 64 walkers 3.2 / 17.0.  The line
 // lies between the closed shells 33 and 57; ftq_autotune times both on the
 // context's own workload.
 constexpr int GREEN_TC_MIN_M = 48;

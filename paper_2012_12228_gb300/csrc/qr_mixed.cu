@@ -733,7 +733,7 @@ cudaError_t launch_tinv_df(ftq_ctx* c) {
 // From this basis size on the T^-1 update runs as a forward substitution with
 // tensor-core updates (green_lu.cu).  Per stabilisation, k_tinv_df against it: M = 57, 640
 // walkers 0.35 / 0.40 ms, M = 123, 256 walkers 0.98 / 0.63, M = 257, 1024 walkers 23.0 /
-// 18.2, M = 515, 64 walkers 18.9 / 7.8.
+// 18.6, M = 515, 64 walkers 18.9 / 7.8.
 constexpr int TINV_LU_MIN_M = 100;
 
 cudaError_t launch_qr_prepiv(ftq_ctx* c) {
