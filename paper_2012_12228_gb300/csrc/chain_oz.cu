@@ -157,7 +157,8 @@ __global__ void __launch_bounds__(NT_OZ, 1) k_chain_oz(const OzArgs p) {
                 }
                 ++li;
             }
-            if (!ok && last >= 0) mbar_wait(&mma_bar[last % NSTAGE], (uint32_t)((last / NSTAGE) & 1));
+            // the MMAs end before TMEM is freed, whichever warp gave up (the epilogue's last wait covers them else)
+            if (last >= 0) mbar_wait(&mma_bar[last % NSTAGE], (uint32_t)((last / NSTAGE) & 1));
         }
     } else if (warp >= W_EPI + W_A) {
         // ------------------------------------------------ digits of Z

@@ -217,11 +217,12 @@ __global__ void __launch_bounds__(NTHREADS_WS, 1) k_chain_tc(const __grid_consta
                     }
                 }
             }
-            if (!ok) {   // abort latched: drain this CTA's own copies and MMAs
+            // drain this CTA's own copies and MMAs: a list walked to its end has waited for every copy, but
+            // another warp may have given up after the last MMAs were issued
+            if (!ok)
                 for (int b = 0; b < NS; ++b)
                     if (last_tma[b] >= 0) mbar_wait(&tma_bar[b], (uint32_t)((last_tma[b] / NS) & 1));
-                if (last_mma >= 0) mbar_wait(&mma_bar[last_mma % NS], (uint32_t)((last_mma / NS) & 1));
-            }
+            if (last_mma >= 0) mbar_wait(&mma_bar[last_mma % NS], (uint32_t)((last_mma / NS) & 1));
         }
     } else if (warp >= NEPI / 32) {
         // ------------------------------------------------ generator warps

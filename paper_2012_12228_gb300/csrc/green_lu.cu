@@ -480,7 +480,8 @@ __global__ void __launch_bounds__(NT_UP, 1) k_lu_update(const UpArgs<T> p, const
                     last = g;
                 }
             }
-            if (!ok && last >= 0) mbar_wait(&mma_bar[last % NST], (uint32_t)((last / NST) & 1));
+            // the MMAs end before TMEM is freed, whichever warp gave up (the epilogue's last wait covers them else)
+            if (last >= 0) mbar_wait(&mma_bar[last % NST], (uint32_t)((last / NST) & 1));
         }
     } else if (warp >= W_EPI + W_A) {
         // ------------------------------------------------ operand B: rows jb.., columns of the tile
