@@ -678,17 +678,23 @@ __global__ void __launch_bounds__(NT_UP, 1) k_lu_update(const UpArgs<T> p, const
         unsigned char* ct = cbuf + (size_t)rr * CROW + part * sizeof(T);
         const int bi = grp;
         int own = 0;                                         // items of this group so far
+        int armed = 0;                                       // loads the mover has put on cfull, one phase each
+        // Once a wait has given up, this warp touches no C tile any more: the load in flight is the last one
+        // armed, so that cfull never has more than one open phase and the buffer more than one writer.
+        bool ok = true;
         for (int it = it0 + grp; it < it1; it += 2, ++own) {
             tile_at(it);
-            if (mover) {
+            if (mover && ok) {
                 if (own > 0) bulk_wait_read();               // the tile stored before has left the buffer
                 fetch();
+                ++armed;
             }
             __syncwarp();
             const uint32_t ph = (uint32_t)(own & 1);
-            bool ok = wait(&tfull[bi], ph);
+            ok = ok && wait(&tfull[bi], ph);
             ok = ok && wait(&cfull[bi], ph);
             if constexpr (F64) ok = ok && wait(&einfo[bi], ph);
+            ok = __all_sync(0xffffffffu, ok);
             tc_fence_after();
             if (ok) {
                 const uint32_t acc = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(bi * ND * OCT);
@@ -759,9 +765,10 @@ __global__ void __launch_bounds__(NT_UP, 1) k_lu_update(const UpArgs<T> p, const
                 bulk_commit();
             }
         }
-        if (mover && own > 0) {
-            // after an abort the last tile may not have been waited for: it must land before the block ends
-            mbar_wait(&cfull[grp], (uint32_t)((own - 1) & 1));
+        if (mover && armed > 0) {
+            // after an abort the last tile armed may not have been waited for (every earlier one has): it
+            // must land before the block ends
+            mbar_wait(&cfull[grp], (uint32_t)((armed - 1) & 1));
             bulk_wait();
         }
     }
