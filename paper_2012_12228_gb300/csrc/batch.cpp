@@ -36,7 +36,7 @@ cudaError_t run_slices(ftq_ctx* b, int n, const double* const* fields) {
         // small bases run a slice's Horner steps in one launch, the others step by step together
         for (int s = 0; s < ns; ++s)
             if (ftq::chain_slice_fits(b->members[s])) {
-                cudaError_t e = ftq::chain_slice(b->members[s]);
+                cudaError_t e = ftq::chain_slice(b->members[s], b);
                 if (e != cudaSuccess) return e;
             }
         for (int s = 0; s < ns; ++s) zin[s] = b->members[s]->Ypl;

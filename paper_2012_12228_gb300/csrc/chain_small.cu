@@ -236,7 +236,8 @@ bool chain_slice_fits(const ftq_ctx* c) {
 }
 
 // exp(V) and the kinetic factors of one slice applied to the mixed chain, in place.
-cudaError_t chain_slice(ftq_ctx* c) {
+// `ruling` sets the bounded waits: the context itself, or the batch it is a member of.
+cudaError_t chain_slice(ftq_ctx* c, const ftq_ctx* ruling) {
     SmallArgs a;
     a.Y = c->Ypl;
     a.Yf = c->Yf;
@@ -251,7 +252,7 @@ cudaError_t chain_slice(ftq_ctx* c) {
     a.NT = (c->M + 15) / 16 * 16;
     a.nslot = c->nslot;
     a.p = c->opts.exp_order;
-    a.wait_limit = c->wait_limit >= 0 ? (long long)c->wait_limit : TC_WAIT_LIMIT;
+    a.wait_limit = ruling->wait_limit >= 0 ? (long long)ruling->wait_limit : TC_WAIT_LIMIT;
     const int KT = 2 * a.Kp / 32;
     const size_t sm = 1024 + (size_t)KT * 2 * (ATILE + a.NT * 128) + sizeof(float2) * a.nslot;
     cudaError_t e = cudaFuncSetAttribute(k_chain_slice, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
