@@ -230,7 +230,10 @@ __global__ void k_slice_summary(const double* __restrict__ rec, int n, double* _
 template <typename T>
 void transpose_g(ftq_ctx* c, const T* G, T* Gt) {
     const unsigned tiles = (unsigned)((c->M + 31) / 32);
-    k_transpose_g<T><<<dim3(tiles, tiles, (unsigned)c->W), dim3(32, 8), 0, c->stream>>>(G, Gt, c->M);
+    const size_t MM = (size_t)c->M * c->M;
+    walker_spans(c->W, [&](size_t w0, int n) {
+        k_transpose_g<T><<<dim3(tiles, tiles, (unsigned)n), dim3(32, 8), 0, c->stream>>>(G + MM * w0, Gt + MM * w0, c->M);
+    });
 }
 
 template <typename T>

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <algorithm>
 #include <cstdint>
 #include <string>
 #include <vector>
@@ -20,6 +21,13 @@ namespace ftq {
 //   [8] d ln|w|/dmu, [9] d arg w/dmu, [10] Re dE, [11] Im dE, [12] Re dN, [13] Im dN
 constexpr int WSTRIDE = 16;
 constexpr int EST_PARTS = 8;      // most blocks that share a walker's estimators
+
+// f(w0, n) for spans [w0, w0 + n) of the walkers: launches with the walkers along y or z of
+// the grid, which end at 65,535.
+template <typename F>
+void walker_spans(int W, F f) {
+    for (int w0 = 0; w0 < W; w0 += 65535) f((size_t)w0, std::min(65535, W - w0));
+}
 
 // Static description of one UEG system (Sec. "Uniform Electron Gas" and
 // "Computational Details").  Built on the host once per context.
@@ -268,6 +276,10 @@ struct LuScales {
     double* lsum;                     // [W] logs of the factors split off
     int* swaps;                       // [W] pivot parity
     int* perm;                        // [W][2][LU_NB_MAX] the panel's permutation
+    LuScales from(size_t w0, int M) const {
+        const size_t o = w0 * M;
+        return {dlb + o, dls + o, drb + o, drs + o, inv + o, lsum + w0, swaps + w0, perm + w0 * 2 * LU_NB_MAX};
+    }
 };
 int lu_ld(int M);
 size_t lu_scal_doubles(int M, int W);

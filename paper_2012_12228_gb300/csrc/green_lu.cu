@@ -964,20 +964,27 @@ cudaError_t lu_solve(ftq_ctx* c, cx<T>* S, const LuScales<T>& sc, int ld) {
     // blocks of at most 128 columns, as even as whole warps allow
     auto blocks = [](int n) { return (n + 127) / 128; };
     auto threads = [&](int n) { return ((n + blocks(n) - 1) / blocks(n) + 31) / 32 * 32; };
-    auto cols = [&](int n) { return dim3((unsigned)((n + threads(n) - 1) / threads(n)), (unsigned)W); };
+    auto cols = [&](int n, int w) { return dim3((unsigned)((n + threads(n) - 1) / threads(n)), (unsigned)w); };
+    const size_t per = (size_t)M * ld;                   // a walker's S
     const int rhs = ld / 2, end = rhs + M;               // columns of the right-hand sides
     for (int jb = 0; jb < M && e == cudaSuccess; jb += NB) {
         const int nb = std::min(NB, M - jb), m = M - jb, c0 = jb + nb;
         c->launches[FTQ_K_GREEN] += 2;
         k_lu_panel<T, NB, MAXT><<<W, (m + 31) / 32 * 32, 0, c->stream>>>(S, sc, c->status, M, ld, jb, nb);
-        k_lu_tri<T, NB, false><<<cols(end - c0), threads(end - c0), 0, c->stream>>>(S, sc, M, ld, jb, nb, c0, end);
+        walker_spans(W, [&](size_t w0, int n) {
+            k_lu_tri<T, NB, false><<<cols(end - c0, n), threads(end - c0), 0, c->stream>>>(
+                S + per * w0, sc.from(w0, M), M, ld, jb, nb, c0, end);
+        });
         e = cudaGetLastError();
         if (e == cudaSuccess) e = launch_update<T>(c, S, ld, jb, nb, c0, M, c0, end);
     }
     for (int jb = (M - 1) / NB * NB; jb >= 0 && e == cudaSuccess; jb -= NB) {
         const int nb = std::min(NB, M - jb);
         c->launches[FTQ_K_GREEN] += 1;
-        k_lu_tri<T, NB, true><<<cols(M), threads(M), 0, c->stream>>>(S, sc, M, ld, jb, nb, rhs, end);
+        walker_spans(W, [&](size_t w0, int n) {
+            k_lu_tri<T, NB, true><<<cols(M, n), threads(M), 0, c->stream>>>(S + per * w0, sc.from(w0, M), M, ld, jb, nb,
+                                                                            rhs, end);
+        });
         e = cudaGetLastError();
         if (e == cudaSuccess) e = launch_update<T>(c, S, ld, jb, nb, 0, jb, rhs, end);
     }
@@ -1026,12 +1033,17 @@ cudaError_t tinv_lu(ftq_ctx* c, const cx<T>* R, const double2* Dp, const int* pe
     const int M = c->M, W = c->W, ld = lu_ld(M), rhs = ld / 2;
     double2* S = c->work;
     double2* dinv = scales_of<double>(c).inv;
-    const dim3 tiles((unsigned)((M + 31) / 32), (unsigned)((M + 31) / 32), (unsigned)W);
+    auto tiles = [&](int n) { return dim3((unsigned)((M + 31) / 32), (unsigned)((M + 31) / 32), (unsigned)n); };
+    const size_t per = (size_t)M * ld, MM = (size_t)M * M;
     k_tinv_diag<T><<<W, 256, 0, c->stream>>>(R, Dp, dinv, c->DR, c->status, M);
-    k_tinv_form<T><<<tiles, 256, 0, c->stream>>>(R, Dp, dinv, perm, c->Tinv, S, M, ld);
+    walker_spans(W, [&](size_t w0, int n) {
+        const size_t o = w0 * M;
+        k_tinv_form<T><<<tiles(n), 256, 0, c->stream>>>(R + MM * w0, Dp ? Dp + o : nullptr, dinv + o, perm + o,
+                                                        c->Tinv + MM * w0, S + per * w0, M, ld);
+    });
     c->launches[FTQ_K_TINV] += 2;
     const int nblk = (M + 127) / 128, nt = ((M + nblk - 1) / nblk + 31) / 32 * 32;
-    const dim3 cols((unsigned)((M + nt - 1) / nt), (unsigned)W);
+    auto cols = [&](int n) { return dim3((unsigned)((M + nt - 1) / nt), (unsigned)n); };
     const size_t sm = sizeof(float4) * (32 * 32 + 32 * (size_t)nt);
     cudaError_t e = cudaGetLastError();
     if (df && e == cudaSuccess)
@@ -1039,14 +1051,20 @@ cudaError_t tinv_lu(ftq_ctx* c, const cx<T>* R, const double2* Dp, const int* pe
                                  (int)(sizeof(float4) * (32 * 32 + 32 * 128)));
     for (int jb = 0; jb < M && e == cudaSuccess; jb += 32) {
         const int nb = std::min(32, M - jb);
-        if (df) k_tinv_tri_df<<<cols, nt, sm, c->stream>>>(S, M, ld, jb, nb, rhs, rhs + M);
-        else k_lu_tri<double, 32, false, false><<<cols, nt, 0, c->stream>>>(S, scales_of<double>(c), M, ld, jb, nb, rhs, rhs + M);
+        walker_spans(W, [&](size_t w0, int n) {
+            double2* Sw = S + per * w0;
+            if (df) k_tinv_tri_df<<<cols(n), nt, sm, c->stream>>>(Sw, M, ld, jb, nb, rhs, rhs + M);
+            else k_lu_tri<double, 32, false, false><<<cols(n), nt, 0, c->stream>>>(
+                Sw, scales_of<double>(c).from(w0, M), M, ld, jb, nb, rhs, rhs + M);
+        });
         c->launches[FTQ_K_TINV] += 1;
         e = cudaGetLastError();
         if (e == cudaSuccess) e = launch_update<double>(c, S, ld, jb, nb, jb + nb, M, rhs, rhs + M, FTQ_K_TINV);
     }
     if (e != cudaSuccess) return e;
-    k_tinv_out<<<tiles, 256, 0, c->stream>>>(S, c->Tinv, c->status, M, ld);
+    walker_spans(W, [&](size_t w0, int n) {
+        k_tinv_out<<<tiles(n), 256, 0, c->stream>>>(S + per * w0, c->Tinv + MM * w0, c->status, M, ld);
+    });
     return cudaGetLastError();
 }
 
@@ -1065,16 +1083,22 @@ cudaError_t launch_green_lu64(ftq_ctx* c, const double2* Y, int k, bool update, 
     const int M = c->M, W = c->W, ld = lu_ld(M);
     const LuScales<double> sc = scales_of<double>(c);
     const double lscale = physical ? 0.0 : left_scale(c, k);
-    const dim3 tiles((unsigned)((M + 31) / 32), (unsigned)((M + 31) / 32), (unsigned)W);
+    auto tiles = [&](int n) { return dim3((unsigned)((M + 31) / 32), (unsigned)((M + 31) / 32), (unsigned)n); };
+    const size_t per = (size_t)M * ld, MM = (size_t)M * M;
     LaunchScope ls(c, FTQ_K_GREEN);
     k_lu_scales<double><<<W, 256, 0, c->stream>>>(c->DR, c->tab.eps, sc, M, lscale, c->sys.mu_T);
-    k_lu_form64<<<tiles, 256, 0, c->stream>>>(Y, c->Tinv, c->work, sc, M, ld);
+    walker_spans(W, [&](size_t w0, int n) {
+        k_lu_form64<<<tiles(n), 256, 0, c->stream>>>(Y + MM * w0, c->Tinv + MM * w0, c->work + per * w0, sc.from(w0, M), M,
+                                                     ld);
+    });
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess)
         e = M <= 384 ? lu_solve<double, 32, 384>(c, c->work, sc, ld) : lu_solve<double, 16, 640>(c, c->work, sc, ld);
     if (e != cudaSuccess) return e;
     c->launches[FTQ_K_GREEN] += 3;      // beside the scope's own: form, G and the tail
-    k_lu_green<double><<<tiles, 256, 0, c->stream>>>(c->work, c->G, sc, M, ld);
+    walker_spans(W, [&](size_t w0, int n) {
+        k_lu_green<double><<<tiles(n), 256, 0, c->stream>>>(c->work + per * w0, c->G + MM * w0, sc.from(w0, M), M, ld);
+    });
     k_lu_tail<double><<<W, 128, 0, c->stream>>>(c->work, c->G, sc, c->wstate, c->status, M, ld,
                                                (double)k * c->sys.dtau, c->opts.constraint, update ? 1 : 0,
                                                physical ? 0 : 1);
@@ -1087,17 +1111,23 @@ cudaError_t launch_green_lu32(ftq_ctx* c, int k, float2* G, double* ws) {
     Planes P;
     P.Kp = c->Kp;
     P.part = (size_t)c->LD * 2 * c->Kp;
-    const dim3 tiles((unsigned)((M + 31) / 32), (unsigned)((M + 31) / 32), (unsigned)W);
+    auto tiles = [&](int n) { return dim3((unsigned)((M + 31) / 32), (unsigned)((M + 31) / 32), (unsigned)n); };
+    const size_t per = (size_t)M * ld, MM = (size_t)M * M;
     LaunchScope ls(c, FTQ_K_GREEN);
     if (!G) G = c->G32;
     k_lu_scales<float><<<W, 256, 0, c->stream>>>(c->DR, c->tab.eps, sc, M, left_scale(c, k), c->sys.mu_T);
-    k_lu_form32<<<tiles, 256, 0, c->stream>>>(c->Ypl, c->Tinv, c->w32, sc, P, 2 * P.part, M, ld);
+    walker_spans(W, [&](size_t w0, int n) {
+        k_lu_form32<<<tiles(n), 256, 0, c->stream>>>(c->Ypl + 2 * P.part * w0, c->Tinv + MM * w0, c->w32 + per * w0,
+                                                     sc.from(w0, M), P, 2 * P.part, M, ld);
+    });
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess)
         e = M <= 640 ? lu_solve<float, 32, 640>(c, c->w32, sc, ld) : lu_solve<float, 16, 1024>(c, c->w32, sc, ld);
     if (e != cudaSuccess) return e;
     c->launches[FTQ_K_GREEN] += 3;      // beside the scope's own: form, G and the tail
-    k_lu_green<float><<<tiles, 256, 0, c->stream>>>(c->w32, G, sc, M, ld);
+    walker_spans(W, [&](size_t w0, int n) {
+        k_lu_green<float><<<tiles(n), 256, 0, c->stream>>>(c->w32 + per * w0, G + MM * w0, sc.from(w0, M), M, ld);
+    });
     k_lu_tail<float><<<W, 128, 0, c->stream>>>(c->w32, G, sc, ws ? ws : c->wstate, c->status, M, ld,
                                               (double)k * c->sys.dtau, c->opts.constraint, 1, 1);
     return cudaGetLastError();

@@ -163,8 +163,12 @@ cudaError_t launch_structure_factor(ftq_ctx* c, double* per_walker_out) {
         LaunchScope ls(c, FTQ_K_ESTIMATORS);
         c->launches[FTQ_K_ESTIMATORS] += 1;
         launch_transpose_g(c, c->G, c->work);
-        k_structure<<<dim3((unsigned)per, (unsigned)W), 512, 0, c->stream>>>(c->G, c->work, c->tab.pair_ptr, c->tab.pair_a,
-                                                                         c->tab.pair_b, c->sq_walker, c->M, nq / 2);
+        const size_t MM = (size_t)c->M * c->M;
+        walker_spans(W, [&](size_t w0, int n) {
+            k_structure<<<dim3((unsigned)per, (unsigned)n), 512, 0, c->stream>>>(
+                c->G + MM * w0, c->work + MM * w0, c->tab.pair_ptr, c->tab.pair_a, c->tab.pair_b,
+                c->sq_walker + w0 * nq, c->M, nq / 2);
+        });
     }
     {
         LaunchScope ls(c, FTQ_K_ESTIMATORS);
