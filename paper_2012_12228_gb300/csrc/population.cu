@@ -235,9 +235,12 @@ cudaError_t launch_population_control(ftq_ctx* c, double xi, int* parent_out) {
     {
         LaunchScope ls(c, FTQ_K_POPULATION);
         const size_t sm = (sizeof(double) + sizeof(int)) * (size_t)W;
-        const bool staged = sm <= 96 * 1024;
-        if (staged && sm > 48 * 1024)
-            cudaFuncSetAttribute(k_comb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        // raised for every size: the 48 KB that need no raising hold the static shared memory too
+        // (W = 4096 takes exactly 48 KB beside it)
+        constexpr size_t limit = 96 * 1024;
+        const bool staged = sm <= limit;
+        cudaError_t e = cudaFuncSetAttribute(k_comb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit);
+        if (e != cudaSuccess) return e;
         k_comb<<<1, 256, staged ? sm : 0, c->stream>>>(c->wstate, c->pc_w, c->pc_cnt, c->pc_parent, c->pc_pairs,
                                                        W, xi, c->status, staged);
     }
@@ -261,10 +264,9 @@ cudaError_t launch_pair_branch(ftq_ctx* c, const double* draws_host, int* parent
                                     c->stream);
     if (e != cudaSuccess) return e;
     const size_t sm = (2 * sizeof(double) + 2 * sizeof(int)) * (size_t)W;
-    if (sm > 48 * 1024) {
-        e = cudaFuncSetAttribute(k_pair_branch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-    }
+    // as in the comb; 8192 walkers at most
+    e = cudaFuncSetAttribute(k_pair_branch, cudaFuncAttributeMaxDynamicSharedMemorySize, 192 * 1024);
+    if (e != cudaSuccess) return e;
     {
         LaunchScope ls(c, FTQ_K_POPULATION);
         k_pair_branch<<<1, 256, sm, c->stream>>>(c->wstate, c->pc_w, c->pc_parent, c->pc_pairs, W, c->status);

@@ -629,7 +629,9 @@ int qr_panel_width(const ftq_ctx* c) {
 cudaError_t launch_qr32(ftq_ctx* c, int nbq) {
     const int M = c->M;
     const size_t smq = 2 * sizeof(float2) * (size_t)M * nbq;
-    static size_t smq_set[3] = {48 * 1024, 48 * 1024, 48 * 1024};
+    // raised from the first launch on: the 48 KB that need no raising hold the static shared memory too
+    // (17 KB with 32 columns)
+    static size_t smq_set[3] = {0, 0, 0};
     const int which = nbq == 32 ? 0 : (nbq == 16 ? 1 : 2);
     cudaError_t e;
     if (smq > smq_set[which]) {
@@ -777,7 +779,7 @@ cudaError_t launch_qr_prepiv(ftq_ctx* c) {
     const bool wide = sizeof(float2) * ((size_t)M * 32 + M) <= 200 * 1024;
     const int QP = wide ? 32 : 16;
     const size_t sm2 = sizeof(float2) * ((size_t)M * QP + M);
-    static size_t sm2_set[2] = {48 * 1024, 48 * 1024};
+    static size_t sm2_set[2] = {0, 0};           // as in launch_qr32
     if (sm2 > sm2_set[wide]) {
         e = wide ? cudaFuncSetAttribute(k_form_q32<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2)
                  : cudaFuncSetAttribute(k_form_q32<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
