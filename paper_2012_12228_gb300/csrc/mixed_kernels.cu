@@ -439,7 +439,7 @@ cudaError_t mixed_qrcp(ftq_ctx* c) {
                                                                           c->M, walker_stride(c), n);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess && c->opts.precision == FTQ_MIXED) e = tc_items_by_rank(c);
+    if (e == cudaSuccess && c->opts.precision == FTQ_MIXED && !chain_slice_fits(c)) e = tc_items_by_rank(c);
     return e;
 }
 
