@@ -352,7 +352,8 @@ int ftq_batch_propagate(ftq_ctx* batch, int n_slices, const double* const* field
  * with tensor-core updates or on CUDA cores, FTQ_Q_GREEN_KERNEL); for a batch
  * every member is tuned.
  * choice / ms: nullable host arrays (one entry per system) receiving the
- * chosen tile count and its time per Horner step.  Uses the scratch buffers
+ * chosen tile count and its time per Horner step (bases up to M = 64 run a
+ * slice's steps in one launch: one tile, and a step's share of the launch).  Uses the scratch buffers
  * of the chain, of the stabilisation and of the estimators; walker state,
  * G(tau) and the status word are not changed. */
 int ftq_autotune(ftq_ctx* ctx, int* choice, float* ms);

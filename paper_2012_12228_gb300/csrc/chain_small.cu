@@ -235,12 +235,12 @@ bool chain_slice_fits(const ftq_ctx* c) {
     return c->M <= 64 && (c->opts.precision == FTQ_MIXED || c->opts.precision == FTQ_MIXED_F64UDT);
 }
 
-// exp(V) and the kinetic factors of one slice applied to the mixed chain, in place.
-// `ruling` sets the bounded waits: the context itself, or the batch it is a member of.
-cudaError_t chain_slice(ftq_ctx* c, const ftq_ctx* ruling) {
+namespace {
+
+cudaError_t launch_slice(ftq_ctx* c, const ftq_ctx* ruling, float* Y, float* Yf) {
     SmallArgs a;
-    a.Y = c->Ypl;
-    a.Yf = c->Yf;
+    a.Y = Y;
+    a.Yf = Yf;
     a.phi = c->phi32;
     a.vidx = c->tab.vidx;
     a.h = c->tab.hf;
@@ -265,6 +265,33 @@ cudaError_t chain_slice(ftq_ctx* c, const ftq_ctx* ruling) {
     LaunchScope ls(c, FTQ_K_CHAIN);
     k_chain_slice<<<std::min(a.W, sms * per_sm), SNT, sm, c->stream>>>(a);
     return cudaGetLastError();
+}
+
+}  // namespace
+
+// exp(V) and the kinetic factors of one slice applied to the mixed chain, in place.
+// `ruling` sets the bounded waits: the context itself, or the batch it is a member of.
+cudaError_t chain_slice(ftq_ctx* c, const ftq_ctx* ruling) { return launch_slice(c, ruling, c->Ypl, c->Yf); }
+
+// Time of one Horner step, from slices of a copy of the chain in the Horner buffers (which
+// small bases do not use otherwise).
+cudaError_t chain_slice_time(ftq_ctx* c, float* ms) {
+    const size_t plane = sizeof(float) * (size_t)c->W * c->LD * 2 * c->Kp;
+    cudaEvent_t e0, e1;
+    cudaEventCreate(&e0);
+    cudaEventCreate(&e1);
+    cudaError_t e = cudaMemcpyAsync(c->zpl[1], c->Yf, plane, cudaMemcpyDeviceToDevice, c->stream);
+    if (e == cudaSuccess) e = launch_slice(c, c, c->zpl[0], c->zpl[1]);      // warm-up
+    if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
+    for (int r = 0; r < 3 && e == cudaSuccess; ++r) e = launch_slice(c, c, c->zpl[0], c->zpl[1]);
+    if (e == cudaSuccess) e = cudaEventRecord(e1, c->stream);
+    if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+    float t = 0.f;
+    if (e == cudaSuccess) e = cudaEventElapsedTime(&t, e0, e1);
+    cudaEventDestroy(e0);
+    cudaEventDestroy(e1);
+    *ms = t / (3.f * c->opts.exp_order);
+    return e;
 }
 
 }  // namespace ftq

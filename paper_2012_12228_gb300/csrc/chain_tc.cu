@@ -844,6 +844,10 @@ cudaError_t tc_batch_items(ftq_ctx* b) {
 // Time one Horner step (scratch output) for each column-tile count and keep
 // the fastest; returns the chosen count.
 cudaError_t tc_autotune(ftq_ctx* c, int* best_nct, float* best_ms) {
+    if (chain_slice_fits(c)) {               // one tile holds every column
+        *best_nct = 1;
+        return chain_slice_time(c, best_ms);
+    }
     int best = c->nct;
     float bms = 1e30f;
     const int n0 = tc_min_nct(c) > 0 ? tc_min_nct(c) : 1;

@@ -301,6 +301,7 @@ cudaError_t oz_chain(ftq_ctx* c);
 // Mixed chain of small bases, a slice in one launch (chain_small.cu).
 bool chain_slice_fits(const ftq_ctx* c);
 cudaError_t chain_slice(ftq_ctx* c, const ftq_ctx* ruling);
+cudaError_t chain_slice_time(ftq_ctx* c, float* ms_per_step);
 
 // Tensor-core chain (chain_tc.cu).
 bool tc_map_3d(void* map, void* base, size_t nx, size_t ny, size_t nz, size_t sy, size_t sz, int bx, int by);

@@ -42,3 +42,26 @@ def test_batch_of_small_members():
     for m, g in zip(b.members, G0):
         assert m.status() == 0 and torch.equal(m.green(), g)
     b.close()
+
+
+def test_autotune_times_the_chain_that_runs():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2012_12228_gb300 as ftq
+    s = SYSTEMS[2]
+    out = []
+    for tune in (False, True):
+        p = ftq.Propagator(s["N"], s["M"], s["rs"], s["theta"], s["dtau"], walkers=9, precision=ftq.FTQ_MIXED)
+        f = torch.from_numpy(gaussian_fields(71, 4, 9, p.n_alpha)).cuda()
+        p.propagate(f[:2].contiguous())
+        if tune:
+            before = p.profile_read()["chain"][1]
+            tiles, ms = p.autotune()
+            assert tiles == 1 and ms > 0
+            assert p.profile_read()["chain"][1] - before == 4      # a warm-up and three timed slices
+            p.set_green_kernel(0)
+        p.propagate(f[2:].contiguous())                   # no stabilisation: the QR panel does not enter
+        out.append((p.green(), p.weights()))
+        assert p.status() == 0
+        p.close()
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
