@@ -10,7 +10,7 @@
 // and 57 bits, written in base 128 as d_0 .. d_7 with |d_j| <= 64 for j >= 1
 // and |d_0| <= 128 (V) or 256 (Z): every digit is a bf16 number.  Products
 // d_i(V) d_j(Z) of one level l = i + j <= 7 are summed in one FP32 accumulator:
-// over at most 512 nonzero real terms a level's sum stays at or below
+// over at most 512 nonzero real terms (256 complex k) a level's sum stays at or below
 // 32768 * 512 = 2^24 for l <= 3 (256 * 128 for l = 0; each further pair adds at
 // most 64 * 64), so it is an exact integer.  From l = 4 on the worst case passes
 // 2^24 by less than 2x, a rounding of one unit there is below 2^-52 of the
@@ -579,7 +579,8 @@ cudaError_t oz_chain(ftq_ctx* c) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit);
     const int grid = std::min(sms, W * a.nrb * a.nct);
     const int tiles = Kp / KC;
-    const int chunks = (M - 1 + CHUNK_K - 1) / CHUNK_K;    // V's diagonal is zero: M - 1 terms per row
+    // whole k tiles per chunk; one chunk also where only V's zero diagonal keeps a row at CHUNK_K terms (M = 257)
+    const int chunks = M - 1 <= CHUNK_K ? 1 : (tiles * KC + CHUNK_K - 1) / CHUNK_K;
     const double* zin = Z0;
     for (int j = p, s = 0; j >= 1 && e == cudaSuccess; --j, ++s) {
         double* zout = Zb[s & 1];

@@ -738,8 +738,8 @@ __global__ void __launch_bounds__(NT_UP, 1) k_lu_update(const UpArgs<T> p, const
 #pragma unroll
                     for (int q = 0; q < 8; ++q) {
                         if constexpr (F64) {
-                            // -2^n for factors scaled by 2^(1079 - e) (a product far below the smallest
-                            // normal number vanishes, an overflow or NaN shows)
+                            // -2^n for factors scaled by 2^(1079 - e): products below about 2^-960, 2^60 above
+                            // the smallest normal number, vanish; an overflow or NaN shows
                             const int ec = (int)col_e[bi][cc + at(q)];
                             const int n = er + ec - 2 * 1079 + 49 + 1023;
                             const uint32_t hw = er == 0x7ff || ec == 0x7ff
