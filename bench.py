@@ -191,7 +191,11 @@ def kernel_model(kind, M, W, precision, green_tc=False):
     Real flops; a complex multiply-add counts 8.  The tensor-core chain runs
     the complex product as three tf32 products (3xTF32), so its tensor work is
     3 x 8 M^3 per walker and its peak is the tf32 dense rate: the measured
-    bf16 GEMM rate times the nominal tf32/bf16 ratio 1.1/2.25."""
+    bf16 GEMM rate times the nominal tf32/bf16 ratio 1.1/2.25.
+
+    green_tc: "lu" for the mixed path's blocked LU with tensor-core updates,
+    4/3 M^3 complex MACs as six bf16 products each; True counts a Gauss-Jordan
+    sweep of 1.5 M^3 as 3xTF32 (records of a kernel that the LU replaced)."""
     fp64 = ("alu", FP64_PEAK_TFLOPS, f"FP64 FMA pipe: {SMS} SMs (device properties) x 2 DFMA/clk x 2 x "
                                       f"{SM_GHZ:.2f} GHz (max SM clock)")
     fp32 = ("alu", FP32_PEAK_TFLOPS, f"FP32 FMA pipe: {SMS} SMs (device properties) x 128 FMA/clk x 2 x "
@@ -209,8 +213,10 @@ def kernel_model(kind, M, W, precision, green_tc=False):
             return (36 * 8.0 * M ** 3 * W,) + digits
         return (8.0 * M ** 3 * W,) + (fp64 if precision == "fp64" else fp32)
     if kind == "green":
-        if green_tc:             # elimination of [Mt^T | B^T] on the tensor cores, counted as 1.5 M^3 complex
-                                 # MACs at tf32 cost (six bf16 products each; the blocked LU needs 4/3 M^3)
+        if green_tc == "lu":
+            return (6 * (8.0 / 3.0 + 8.0) * M ** 3 * W, "tensor", bf16,
+                    f"bf16 dense = {bf16:.1f} TFLOP/s (MEASURED_PEAKS.json), six bf16 products per FP32 one")
+        if green_tc:
             return (3 * 12.0 * M ** 3 * W,) + tf32
         if precision == "fp64" and 48 <= M <= 640:
             return (36 * (8.0 / 3.0 + 8.0) * M ** 3 * W,) + digits
@@ -221,9 +227,11 @@ def kernel_model(kind, M, W, precision, green_tc=False):
             return ((16.0 / 3.0 + 16.0 / 3.0 + 4.0) * M ** 3 * W,) + fp64
         return ((16.0 / 3.0) * M ** 3 * W,) + fp32          # FP32 Householder of Y Pi (Q: bridge class)
     if kind == "tinv":           # T^-1 <- T^-1 Pi U^-1: a triangular solve with M right-hand sides
-        if M >= 100:
+        if precision != "mixed":
+            return (4.0 * M ** 3 * W,) + fp64
+        if M >= 100:             # digit updates on the tensor cores
             return (36 * 4.0 * M ** 3 * W,) + digits
-        return (4.0 * M ** 3 * W,) + fp64
+        return (48.0 * M ** 3 * W,) + fp32     # double-FP32: 48 FP32 instructions per complex MAC, 2 flop each
     return None
 
 
@@ -344,7 +352,7 @@ def measure_path(ftq, torch, dev, precision, W, steps, warmup, world, rank, barr
     prof = {k: {"ms": after[k][0], "n_timed": ops.get(k, after[k][1] - before[k][1]) if after[k][0] > 0 else 0}
             for k in after}
     out["kernel_ms_per_step"] = {k: v["ms"] for k, v in prof.items() if v["ms"] > 0}
-    out["roofline"] = roofline(prof, M, W, precision, green_tc=prop.query("GREEN_KERNEL") == 1)
+    out["roofline"] = roofline(prof, M, W, precision, green_tc="lu" if prop.query("GREEN_KERNEL") == 1 else False)
     out["device_status"] = prop.status()
     out["slice_average"] = measure_tracking(torch, prop, stream, fields)
     out["population_control"] = measure_comb(torch, prop, stream, precision, fields)
@@ -473,7 +481,7 @@ def ragged_roofline(b, fl, stab, ctxs):
     model = None
     for sd, m in zip(RAGGED, b.members):
         per_block = {"chain": 6 * stab, "green": stab, "qrcp": 1, "tinv": 1}.get(dom, 0)
-        mm = kernel_model(dom, m.M, m.W, "mixed", m.query("GREEN_KERNEL") == 1)
+        mm = kernel_model(dom, m.M, m.W, "mixed", "lu" if m.query("GREEN_KERNEL") == 1 else False)
         if mm is None or per_block == 0:
             model = None
             break
