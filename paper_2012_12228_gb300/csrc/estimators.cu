@@ -12,10 +12,10 @@
 // k_est_walkers: persistent blocks over walkers, or over parts of them when there
 // are fewer walkers than blocks (a walker's G stays in L2 while it is worked on); a warp per slot for rho; for Lambda a warp
 // per work unit = 32 consecutive pairs (a, d) of one +Q transfer (one per
-// lane), looping over all pairs (b, c) of that transfer: P_ab = delta_ab -
-// G[b][a] is read from row b of G and P_cd = delta_cd - G[d][c] from row c
-// of G^T (written by k_transpose_g), so the 32 lanes of a load touch
-// neighbouring columns of one row, which needs few sectors.  With FP32 G
+// lane), looping over all pairs (b, c) of that transfer (exchange.cuh): G[b][a]
+// is read from row b of G and G[d][c] from row c of G^T (written by
+// k_transpose_g), so the 32 lanes of a load touch neighbouring columns of
+// one row, which needs few sectors; the deltas of P are added once per pair.  With FP32 G
 // each lane accumulates v_Q times its partial sum as a compensated float
 // pair (two-sum), so no FP64 instruction runs per unit; with complex128 G the
 // products and sums are FP64 (the FP64 pipe bounds that variant).

@@ -17,7 +17,8 @@
 //                under one power of two per row of A and per column of B (see
 //                chain_oz.cu; the level sums over 2 NB terms stay below 2^22).
 //                FP32 digits with exact sums gave the same errors of G and ln det to
-//                two figures and took 1.6 times as long.
+//                two figures and took 1.6 times as long (only behind a stabilisation at M = 515
+//                does the truncation of the level sums show: ln det 7e-6 off, 4e-6 with FP64 sums).
 // Everything but the panel is spread over (walker, tile) items, so that few
 // walkers fill the chip as well as many, and no walker's serial chain of panels
 // holds an SM.
@@ -113,10 +114,11 @@ __global__ void __launch_bounds__(256) k_lu_form64(const double2* __restrict__ Y
     }
 }
 
-// t s for FP64 t and s = b r in FP32 pairs, about 2^-24 relative in all.  It is
-// integer and FP32 work only: with three FP64 multiplications and four
-// conversions per entry the kernel ran at the FP64 pipe's rate (1.09 ms at
-// M = 257, 1024 walkers).
+// t s for FP64 t and s = b r in FP32 pairs (48 bits), rounded to FP32 once: the number that
+// an FP64 product rounds to, but for rounding ties (none of 4 million products above 1e-33
+// differs; below, the pairs' low words run out of exponents).  It is integer and FP32
+// work only: with three FP64 multiplications and four conversions per entry the kernel ran at
+// the FP64 pipe's rate (1.09 ms at M = 257, 1024 walkers).
 __device__ __forceinline__ float scaled(double t, float sh, float sl) {
     const df2 v = df_split_int(t);
     return fmaf(v.h, sh, fmaf(v.h, sl, v.l * sh));
@@ -362,8 +364,9 @@ __global__ void __launch_bounds__(128) k_tinv_tri_df(double2* __restrict__ S, in
 // numbers of 16 rows and meet no bank conflicts in the C tile) and k tiles
 // [Re (16) | Im (16)], as in chain_oz.cu.  Stores of operand digits alternate
 // between the two rows (A) and the two 8-byte halves (B) over the lanes for the
-// same reason: the kernel is bound by shared-memory wavefronts (64% of the pipe
-// with conflicts), not by the tensor pipe (8%) or DRAM (30%).
+// same reason.  What bounds the FP32 items is shared-memory wavefronts (63% of the
+// pipe; tensor pipe 17%, DRAM 44%, at M = 257, 304 walkers), the complex128 ones the FP64 pipe
+// and the integer ALU of the epilogue (49% each).
 template <typename T> struct UpCfg;
 template <> struct UpCfg<double> { static constexpr int ND = 8, OCT = 32, NST = 2; };
 template <> struct UpCfg<float> { static constexpr int ND = 3, OCT = 64, NST = 4; };
