@@ -9,8 +9,8 @@
 // is the trace of a product of two gathered blocks, tr(XY) = tr(YX)), so only
 // the half-space transfers are summed and counted twice.
 //
-// k_est_walkers: persistent blocks over walkers, or over parts of them when there
-// are fewer walkers than blocks (a walker's G stays in L2 while it is worked on); a warp per slot for rho; for Lambda a warp
+// k_est_walkers: persistent blocks over walkers or over equal parts of them (est_parts; a
+// walker's G stays in L2 while it is worked on); a warp per slot for rho; for Lambda a warp
 // per work unit = 32 consecutive pairs (a, d) of one +Q transfer (one per
 // lane), looping over all pairs (b, c) of that transfer (exchange.cuh): G[b][a]
 // is read from row b of G and G[d][c] from row c of G^T (written by
@@ -21,6 +21,7 @@
 // products and sums are FP64 (the FP64 pipe bounds that variant).
 // T = double2 reads a complex128 G; T = float2 the FP32 G of the mixed
 // path's slices.
+#include <algorithm>
 #include <cmath>
 
 #include "block_reduce.cuh"
@@ -80,13 +81,13 @@ __global__ void __launch_bounds__(1024) k_est_walkers(const T* __restrict__ G, c
     double2* rho = reinterpret_cast<double2*>(smem_raw);     // [2 nqh + 1]
     __shared__ double2 shc[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int nslot = 2 * nqh + 1;
     for (int item = blockIdx.x; item < W * nparts; item += gridDim.x) {
         const int w = item / nparts, part = item % nparts;
         const T* Gw = G + (size_t)w * M * M;
         const T* Gt = Gtr + (size_t)w * M * M;
-        // the first part of a walker also takes everything but the exchange sum
-        for (int sl = 1 + warp; sl < nslot && part == 0; sl += nw) {
+        // both slots of every nparts-th transfer (the sums over a alone are the first part's)
+        for (int s = warp; part + (s >> 1) * nparts < nqh; s += nw) {
+            const int sl = 1 + 2 * (part + (s >> 1) * nparts) + (s & 1);
             double2 r = make_double2(0.0, 0.0);
             for (int e = pptr[sl] + lane; e < pptr[sl + 1]; e += 32) r = r + to_d(pel(Gw, M, pa[e], pb[e]));
             r = warp_sum_d(r);
@@ -102,8 +103,15 @@ __global__ void __launch_bounds__(1024) k_est_walkers(const T* __restrict__ G, c
             nsum = nsum + p * 2.0;
             e1 = e1 + p * ksq[a];
         }
-        for (int q = threadIdx.x; q < nqh && part == 0; q += blockDim.x) e2 = e2 + cmul(rho[1 + 2 * q], rho[2 + 2 * q]) * (4.0 * vq[q]);
-        for (int u = warp * nparts + part; u < nunits; u += nw * nparts) {
+        for (int q = part + (int)threadIdx.x * nparts; q < nqh; q += blockDim.x * nparts)
+            e2 = e2 + cmul(rho[1 + 2 * q], rho[2 + 2 * q]) * (4.0 * vq[q]);
+        // The units shorten along the list: every other round of the warps of all parts runs
+        // backwards, so that each warp, and with it each part, gets about the same work (complex128,
+        // M = 171, one block per walker: 2.13 -> 1.38 ms).
+        const int round = nw * nparts, t = warp * nparts + part;
+        for (int u0 = 0, back = 0; u0 < nunits; u0 += round, back ^= 1) {
+            const int u = u0 + (back ? round - 1 - t : t);
+            if (u >= nunits) continue;
             const int4 un = units[u];                  // slot pairs [x, y), chunk from z, v_Q index w
             const int f = un.z + lane;
             const bool on = f < un.y;
@@ -236,6 +244,31 @@ void transpose_g(ftq_ctx* c, const T* G, T* Gt) {
     });
 }
 
+// Parts of a walker: those that leave the least to the busiest SM.  Blocks take items in
+// turn and neighbouring blocks share an SM, so its share is ceil(W n / blocks) items per
+// block, each 1 / n of a walker and a fixed cost: 190 / M^2 of a walker's time for complex128
+// G, 12 / M + 250 / M^2 for FP32 G.  A part has at least one unit for most warps.  Where the walkers under way read more than 300 MB, twice the L2 and
+// more, fewer of them at a time are worth a quarter (complex128, M = 389, 152 walkers: 19.0 ms
+// with one part, 11.5 with six).  A split that filled its rounds badly was slower than none:
+// FP32, M = 57, 110 walkers in two parts 0.168 ms against 0.100 in one; complex128, M = 147,
+// 152 walkers in eight parts 2.07 ms against 1.57 (now 1.00), M = 257, 128 walkers 5.09 (now
+// 3.30 in seven parts).
+int est_parts(int W, int M, int nunits, int nwarp, int sms, int per_sm, bool f32) {
+    const double fixed = f32 ? 12.0 / M + 250.0 / ((double)M * M) : 190.0 / ((double)M * M);
+    const double bytes = (f32 ? 16.0 : 32.0) * M * M;                  // G and G^T
+    const int blocks = per_sm * sms;
+    int best = 1;
+    double low = 1e300;
+    for (int n = 1; n <= EST_PARTS && (n - 1) * nwarp < nunits; ++n) {
+        const long long items = (long long)W * n;
+        const double rounds = (double)((items + blocks - 1) / blocks) * (items <= sms ? 1 : per_sm);
+        const double walkers = std::min((double)W, (double)blocks / n);
+        const double cost = rounds / n * (1.0 + n * fixed) * (walkers * bytes > 300e6 ? 1.25 : 1.0);
+        if (cost < low) { low = cost; best = n; }
+    }
+    return best;
+}
+
 template <typename T>
 cudaError_t launch_est_walkers(ftq_ctx* c, const T* G) {
     const int nqh = c->sys.nq_half;
@@ -257,13 +290,7 @@ cudaError_t launch_est_walkers(ftq_ctx* c, const T* G) {
     // the L2; complex128 G (FP64-pipe bound): two 512-thread blocks per SM
     const int nthr = f32 ? 1024 : 512;
     const int per_sm = f32 ? 1 : 2;
-    // fewer walkers than four rounds of blocks (FP32 G: than blocks, since the loads of a
-    // split walker's G come from L2 more than once): a walker's exchange units are split
-    // (M = 257, 128 walkers, complex128: 5.8 ms with one block each, 5.0 split)
-    const int target = f32 ? sms : 4 * per_sm * sms;
-    int nparts = c->W < target ? (target + c->W - 1) / c->W : 1;
-    nparts = nparts > EST_PARTS ? EST_PARTS : nparts;
-    if (nparts > c->tab.neplus / 64) nparts = c->tab.neplus < 64 ? 1 : c->tab.neplus / 64;   // small bases: one block
+    const int nparts = est_parts(c->W, M, c->tab.neplus, nthr / 32, sms, per_sm, f32);
     const int grid = c->W * nparts < per_sm * sms ? c->W * nparts : per_sm * sms;
     LaunchScope ls(c, FTQ_K_ESTIMATORS);
     // G^T into the complex128 work buffer (scratch between calls; it holds a
