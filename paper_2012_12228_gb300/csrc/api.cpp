@@ -220,6 +220,11 @@ int ftq_init_ueg(ftq_ctx** out, int N, int M, double rs, double theta, double mu
             for (int e = s.pair_ptr[sl]; e < s.pair_ptr[sl + 1]; e += 32)
                 eplus.push_back(make_int4(s.pair_ptr[sl], s.pair_ptr[sl + 1], e, (sl - 1) >> 1));
         c->tab.neplus = (int)eplus.size();
+        for (int q = 0; q < s.nq_half; ++q) {
+            const int pairs = s.pair_ptr[2 + 2 * q] - s.pair_ptr[1 + 2 * q];
+            if (pairs > 16) c->sq_whole = q + 1;
+            if (pairs > 8) c->sq_half = q + 1;
+        }
         chk(upload(c, &c->tab.eplus, eplus));
     }
     if (e == cudaSuccess && (opts->precision == FTQ_MIXED || opts->precision == FTQ_MIXED_F64UDT)) {

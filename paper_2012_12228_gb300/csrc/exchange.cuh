@@ -6,15 +6,13 @@
 
 namespace ftq {
 
-// Lane sum for the pairs [first, end) of the transfer and this lane's pair (al, dl).
-// Since a - d = b - c, the Kronecker deltas meet only at (b, c) = (a, d), and both do:
-// the loop sums the products G[b][a] G[d][c] alone, and 1 - G[a][a] - G[d][d] is added
-// once.  G^T is read beside G so that the 32 lanes of a load touch neighbouring
-// columns of one row; four partial sums keep eight loads in flight per lane.
+// Lane sum of the products G[b][a] G[d][c] for the pairs [first, end) of the transfer and
+// this lane's pair (al, dl).  G^T is read beside G so that the 32 lanes of a load touch
+// neighbouring columns of one row; four partial sums keep eight loads in flight per lane.
 template <typename T>
-__device__ __forceinline__ T exchange_unit(const T* __restrict__ Gw, const T* __restrict__ Gt, int M,
-                                           const int* __restrict__ pa, const int* __restrict__ pb, int first, int end,
-                                           int al, int dl) {
+__device__ __forceinline__ T exchange_products(const T* __restrict__ Gw, const T* __restrict__ Gt, int M,
+                                               const int* __restrict__ pa, const int* __restrict__ pb, int first,
+                                               int end, int al, int dl) {
     const T* gcol = Gw + al;                   // G[b][al] = gcol[b * M]
     const T* tcol = Gt + dl;                   // G[dl][c] = G^T[c][dl] = tcol[c * M]
     T acc[4];
@@ -33,7 +31,16 @@ __device__ __forceinline__ T exchange_unit(const T* __restrict__ Gw, const T* __
         for (int u = 0; u < 4; ++u) acc[u] = cfma(x[u], y[u], acc[u]);
     }
     for (; g < end; ++g) acc[0] = cfma(gcol[pa[g] * M], tcol[pb[g] * M], acc[0]);
-    T r = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+    return (acc[0] + acc[1]) + (acc[2] + acc[3]);
+}
+
+// The same with the deltas.  Since a - d = b - c they meet only at (b, c) = (a, d), and both
+// do: 1 - G[a][a] - G[d][d] is added once.
+template <typename T>
+__device__ __forceinline__ T exchange_unit(const T* __restrict__ Gw, const T* __restrict__ Gt, int M,
+                                           const int* __restrict__ pa, const int* __restrict__ pb, int first, int end,
+                                           int al, int dl) {
+    T r = exchange_products<T>(Gw, Gt, M, pa, pb, first, end, al, dl);
     const T ga = Gw[al * M + al], gd = Gw[dl * M + dl];
     r.x += 1 - ga.x - gd.x;
     r.y -= ga.y + gd.y;

@@ -149,6 +149,7 @@ struct ftq_ctx {
     int* pc_pairs = nullptr;
     bool resampled = false;       // a comb happened since the last reset
     // structure factor: per-walker <rho(Q) rho(-Q)>, weights, reduced sums (allocated on first use)
+    int sq_whole = 0, sq_half = 0;   // first transfers from which none has more than 16, more than 8 pairs
     double2* sq_walker = nullptr;
     double2* sq_w = nullptr;
     double* sq_out = nullptr;

@@ -15,59 +15,88 @@
 namespace ftq {
 namespace {
 
-// P_ab = <a+_a a_b> = delta_ab - G_ba
-__device__ __forceinline__ double2 pel_s(const double2* Gw, int M, int a, int b) {
-    const double2 g = Gw[(size_t)b * M + a];
-    return make_double2((a == b ? 1.0 : 0.0) - g.x, -g.y);
+// Totals over groups of GS lanes of eight values: the lanes halve the list as they halve the
+// distance, seven to nine additions for eight values (a warp's FP64 addition takes 16 cycles
+// of the SM).  Lane i GS / 8 of a group holds its total of value i.
+template <int GS>
+__device__ __forceinline__ double group_totals(double (&v)[8]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int n = 4, o = GS / 2; n >= 1; n >>= 1, o >>= 1)
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const bool up = lane & o;
+            const double give = up ? v[i] : v[i + n];
+            v[i] = (up ? v[i + n] : v[i]) + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+#pragma unroll
+    for (int o = GS / 16; o >= 1; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    return v[0];
 }
 
-__device__ __forceinline__ double2 warp_total(double2 v) {
-    for (int o = 16; o > 0; o >>= 1) {
-        v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
-        v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+// The transfers q .. q + 32 / GS - 1 below end_q, one per group of GS lanes; with GS < 32 none
+// has more than GS pairs.
+template <int GS>
+__device__ __forceinline__ void structure_task(const double2* Gw, const double2* Gt, const int* __restrict__ pptr,
+                                               const int* __restrict__ pa, const int* __restrict__ pb, double2* out,
+                                               int M, int q, int end_q) {
+    const int lane = threadIdx.x & 31, gl = lane & (GS - 1), g0 = lane - gl;
+    q += lane / GS;
+    const bool live = q < end_q;
+    const int first = live ? pptr[1 + 2 * q] : 0, end = live ? pptr[2 + 2 * q] : 0;
+    double2 rp = make_double2(0.0, 0.0), rm = rp, sa = rp, sb = rp, x = rp;
+    for (int e0 = first; e0 < end; e0 += GS) {
+        const int e = e0 + gl;
+        const bool on = e < end;
+        const int a = on ? pa[e] : 0, d = on ? pb[e] : 0;
+        const double2 t = exchange_products<double2>(Gw, Gt, M, pa, pb, first, end, a, d);
+        if (on) {
+            x = x + t;
+            rp = rp - Gw[(size_t)d * M + a];                 // P_ad, a != d
+            rm = rm - Gw[(size_t)a * M + d];
+            sa = sa + Gw[(size_t)a * M + a];
+            sb = sb + Gw[(size_t)d * M + d];
+        }
     }
-    return v;
+    __syncwarp();
+    const double2 u = sb - x, v = sa - x;
+    double all[8] = {rp.x, rp.y, rm.x, rm.y, u.x, u.y, v.x, v.y};
+    const double t = group_totals<GS>(all);
+    auto get = [&](int i) { return __shfl_sync(0xffffffffu, t, g0 + i * (GS / 8)); };
+    const double2 p = make_double2(2.0 * get(0), 2.0 * get(1)), m = make_double2(2.0 * get(2), 2.0 * get(3));
+    const int sl = gl & 1;                                   // lanes 0 and 1 of a group: slots +Q and -Q
+    const double2 o = make_double2(get(4 + 2 * sl), get(5 + 2 * sl));
+    if (live && gl < 2) out[2 * q + gl] = cmul(p, m) + o * 2.0;
 }
 
-// A warp per walker and half-space transfer q (slots 1 + 2 q and 2 + 2 q, whose
-// pairs are each other's reversed): rho and D of both, and Lambda once, since
-// Lambda_-Q = Lambda_Q.  The short transfers have the most pairs and come first;
-// the warps of a walker's blocks take them in turn.  The FP64 pipe bounds it (four
-// DFMA per exchange term).
-__global__ void __launch_bounds__(512) k_structure(const double2* __restrict__ G, const double2* __restrict__ Gtr,
+// A group of lanes per walker and half-space transfer q (slots 1 + 2 q and 2 + 2 q, whose
+// pairs are each other's reversed): both slots at once, since Lambda_-Q = Lambda_Q.
+// With the deltas summed over the n pairs (a, d) of Q,
+//   Lambda / 2 = X + n - A - B,  D_Q / 2 = n - A,  D_-Q / 2 = n - B,
+// X the products of the exchange sum, A = sum G_aa, B = sum G_dd: n drops out, and
+// Gamma + 2 (B - X), Gamma + 2 (A - X) are left.
+// The FP64 pipe bounds it (four DFMA per exchange term, 16 cycles of an SM each for a whole
+// warp), so lanes must not idle: the transfers up to `whole` take a warp each, those up to
+// `half` (at most 16 pairs) share one by twos, the rest (at most 8) by fours.  The short
+// transfers have the most pairs and come first; the warps of a walker's blocks take the
+// tasks in turn.  Whole calls, before both signs shared a sum, then with a warp per transfer,
+// and now: M = 33, 1216 walkers 0.72, 1.31 and 0.61 ms; M = 57, 608 walkers 0.82, 1.17 and
+// 0.63; M = 257, 128 walkers 14.5, 5.2 and 3.7.  Two blocks per SM at 64 registers, with
+// spills, beat one at 96 (M = 171, 152 walkers 1.56 against 2.11 ms).
+__global__ void __launch_bounds__(512, 2) k_structure(const double2* __restrict__ G, const double2* __restrict__ Gtr,
                                                   const int* __restrict__ pptr, const int* __restrict__ pa,
                                                   const int* __restrict__ pb, double2* __restrict__ out, int M,
-                                                  int nqh) {
-    const int w = blockIdx.y, lane = threadIdx.x & 31;
+                                                  int nqh, int whole, int half) {
+    const int w = blockIdx.y;
     const int warp = blockIdx.x + gridDim.x * (threadIdx.x >> 5), nw = gridDim.x * (blockDim.x >> 5);
     const double2* Gw = G + (size_t)w * M * M;
     const double2* Gt = Gtr + (size_t)w * M * M;
-    for (int q = warp; q < nqh; q += nw) {
-        const int first = pptr[1 + 2 * q], end = pptr[2 + 2 * q];
-        double2 rp = make_double2(0.0, 0.0), rm = rp, dp = rp, dm = rp, lam = rp;
-        for (int e0 = first; e0 < end; e0 += 32) {
-            const int e = e0 + lane;
-            const bool on = e < end;
-            const int a = on ? pa[e] : 0, d = on ? pb[e] : 0;
-            const double2 x = exchange_unit<double2>(Gw, Gt, M, pa, pb, first, end, a, d);
-            if (on) {
-                lam = lam + x;
-                rp = rp + pel_s(Gw, M, a, d);
-                rm = rm + pel_s(Gw, M, d, a);
-                dp = dp + pel_s(Gw, M, a, a);
-                dm = dm + pel_s(Gw, M, d, d);
-            }
-        }
-        lam = warp_total(lam);
-        rp = warp_total(rp);
-        rm = warp_total(rm);
-        dp = warp_total(dp);
-        dm = warp_total(dm);
-        if (lane == 0) {
-            const double2 g = cmul(rp * 2.0, rm * 2.0) - lam * 2.0;
-            out[((size_t)w * nqh + q) * 2] = g + dp * 2.0;
-            out[((size_t)w * nqh + q) * 2 + 1] = g + dm * 2.0;
-        }
+    double2* o = out + (size_t)w * nqh * 2;
+    const int twos = (half - whole + 1) / 2, tasks = whole + twos + (nqh - half + 3) / 4;
+    for (int t = warp; t < tasks; t += nw) {
+        if (t < whole) structure_task<32>(Gw, Gt, pptr, pa, pb, o, M, t, whole);
+        else if (t < whole + twos) structure_task<16>(Gw, Gt, pptr, pa, pb, o, M, whole + 2 * (t - whole), half);
+        else structure_task<8>(Gw, Gt, pptr, pa, pb, o, M, half + 4 * (t - whole - twos), nqh);
     }
 }
 
@@ -154,12 +183,13 @@ cudaError_t launch_structure_factor(ftq_ctx* c, double* per_walker_out) {
         if (e != cudaSuccess) return e;
     }
     {
-        // enough 512-thread blocks for four rounds of two per SM (M = 257, 128 walkers: one 256-thread
-        // block per walker with both signs of Q summed took 14.6 ms)
+        // enough 512-thread blocks for four rounds of two per SM
         int dev = 0, sms = 1;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const int per = std::max(1, std::min((8 * sms + W - 1) / W, (nq / 2 + 15) / 16));
+        const int nqh = nq / 2, whole = c->sq_whole, half = c->sq_half;
+        const int tasks = whole + (half - whole + 1) / 2 + (nqh - half + 3) / 4;
+        const int per = std::max(1, std::min((8 * sms + W - 1) / W, (tasks + 15) / 16));
         LaunchScope ls(c, FTQ_K_ESTIMATORS);
         c->launches[FTQ_K_ESTIMATORS] += 1;
         launch_transpose_g(c, c->G, c->work);
@@ -167,7 +197,7 @@ cudaError_t launch_structure_factor(ftq_ctx* c, double* per_walker_out) {
         walker_spans(W, [&](size_t w0, int n) {
             k_structure<<<dim3((unsigned)per, (unsigned)n), 512, 0, c->stream>>>(
                 c->G + MM * w0, c->work + MM * w0, c->tab.pair_ptr, c->tab.pair_a, c->tab.pair_b,
-                c->sq_walker + w0 * nq, c->M, nq / 2);
+                c->sq_walker + w0 * nq, c->M, nqh, whole, half);
         });
     }
     {
