@@ -259,9 +259,9 @@ __global__ void __launch_bounds__(1024) k_qrcp(const double2* __restrict__ Yin, 
 // then ln S_k = 2 (ln det_k - ln det_{k-1}) and the weight (Eqs. import,
 // phimport, theta).
 //
-// L lanes share a column of the LU's updates and a row of the solves: four for the
-// small bases, where a lane per row left half of a block's lanes idle and the
-// sums' latency exposed.
+// L lanes share a column of the LU's updates and a row of the solves: more than one for
+// the small bases, where a lane per row left half of a block's lanes idle and the
+// sums' latency exposed (green_lanes).
 template <int L>
 __device__ __forceinline__ double2 lane_sum(double2 s) {
 #pragma unroll
@@ -407,13 +407,28 @@ __global__ void __launch_bounds__(1024) k_green(const double2* __restrict__ Y, c
 }
 
 // The one-block factorisations of bases below lu64_supported's keep their matrices in
-// shared memory (two for G, three for the QRCP; at most 106 KB at M = 47).  Per launch
-// at M = 33, 300 walkers: G 378 -> 350 us (314 with four lanes per row), QRCP 670 -> 618 us
-// (468 with two lanes per column).
+// shared memory (two for G, three for the QRCP; at most 106 KB at M = 47) while an SM has
+// four walkers at most: their time is latency then.  Per launch at M = 33, 300 walkers: G 378 ->
+// 350 us (314 with four lanes per row), QRCP 670 -> 618 us (468 with two lanes per column).
+// With more walkers an SM is filled by other blocks: one lane per row or column and the
+// matrices in L2, so that more blocks fit (G of ten slices, this and the other: M = 27, 2432
+// walkers 7.7 / 13.1 ms, M = 33 18.1 / 22.2, 608 walkers 5.1 / 5.7; a QRCP of M = 33, 2432 walkers
+// 4.9 / 5.4 ms).
 constexpr int SMEM_M = 47;
 
-size_t fact_smem(int M, size_t vectors, int matrices) {
-    return M <= SMEM_M ? ((vectors + 15) & ~(size_t)15) + sizeof(double2) * matrices * (size_t)M * M : vectors;
+bool in_smem(const ftq_ctx* c) { return c->M <= SMEM_M && c->W <= 4 * sm_count(); }
+
+size_t fact_smem(const ftq_ctx* c, size_t vectors, int matrices) {
+    return in_smem(c) ? ((vectors + 15) & ~(size_t)15) + sizeof(double2) * matrices * (size_t)c->M * c->M : vectors;
+}
+
+// Lanes per row of k_green: four while an SM has one walker and a half, two up to four (M = 33, ten
+// slices, 304 walkers 3.15 ms with four lanes, 2.84 with two; 608 walkers 5.73 and 4.66); four
+// also where they fit one warp.  Larger bases (M > 640): one.
+int green_lanes(const ftq_ctx* c) {
+    if (c->M > SMEM_M) return 1;
+    const int sms = sm_count();
+    return 4 * c->M <= 32 || 2 * c->W <= 3 * sms ? 4 : (c->W <= 4 * sms ? 2 : 1);
 }
 
 int fact_threads(int M) {
@@ -465,8 +480,10 @@ cudaError_t launch_chain(ftq_ctx* c) {
 
 cudaError_t launch_qrcp64(ftq_ctx* c, const double2* Yin, double2* Qout) {
     const int M = c->M;
-    const size_t sm = fact_smem(M, (sizeof(double) + sizeof(int)) * M, 3);
-    const int nt = std::min(1024, 2 * fact_threads(M));      // two lanes per column
+    const bool small = in_smem(c);
+    const size_t sm = fact_smem(c, (sizeof(double) + sizeof(int)) * M, 3);
+    const int lanes = M > SMEM_M || small ? 2 : 1;           // per column
+    const int nt = std::min(1024, lanes * fact_threads(M));
     if (sm > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k_qrcp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
@@ -475,7 +492,7 @@ cudaError_t launch_qrcp64(ftq_ctx* c, const double2* Yin, double2* Qout) {
     double2* R = lu ? c->zbuf[1] : c->work;      // S of the T^-1 update takes the work buffer
     LaunchScope ls(c, FTQ_K_QRCP);
     k_qrcp<<<c->W, nt, sm, c->stream>>>(Yin, Qout, R, c->work2, c->DR, c->Tinv, c->hh, c->htau,
-                                       c->wstate, c->status, lu ? c->perm : nullptr, M, M <= SMEM_M ? 1 : 0);
+                                       c->wstate, c->status, lu ? c->perm : nullptr, M, small ? 1 : 0);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && lu) e = launch_tinv_lu64(c, R, c->perm);
     return e;
@@ -500,16 +517,16 @@ cudaError_t launch_green64(ftq_ctx* c, const double2* Y, int k, bool update, boo
     const int M = c->M;
     if (c->opts.low_rank_threshold > 0.0) return launch_green_lr(c, Y, k, update, physical);
     if (lu64_supported(M)) return launch_green_lu64(c, Y, k, update, physical);
-    const size_t sm = fact_smem(M, (2 * sizeof(double2) + 3 * sizeof(double) + sizeof(int)) * M, 2);
+    const size_t sm = fact_smem(c, (2 * sizeof(double2) + 3 * sizeof(double) + sizeof(int)) * M, 2);
     const double lscale = physical ? 0.0 : left_scale(c, k);
-    const bool small = M <= SMEM_M;
-    auto kernel = small ? k_green<4> : k_green<1>;
-    const int nt = small ? (4 * M + 31) / 32 * 32 : fact_threads(M);
+    const int L = green_lanes(c);
+    auto kernel = L == 4 ? k_green<4> : (L == 2 ? k_green<2> : k_green<1>);
+    const int nt = L > 1 ? (L * M + 31) / 32 * 32 : fact_threads(M);
     if (sm > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     LaunchScope ls(c, FTQ_K_GREEN);
     kernel<<<c->W, nt, sm, c->stream>>>(Y, c->Tinv, c->DR, c->work, c->work2, c->G, c->tab.eps, c->wstate,
                                        c->status, M, lscale, c->sys.mu_T, c->opts.constraint, update ? 1 : 0,
-                                       physical ? 0 : 1, (double)k * c->sys.dtau, small ? 1 : 0);
+                                       physical ? 0 : 1, (double)k * c->sys.dtau, in_smem(c) ? 1 : 0);
     return cudaGetLastError();
 }
 

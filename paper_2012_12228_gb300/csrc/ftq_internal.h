@@ -22,6 +22,13 @@ namespace ftq {
 constexpr int WSTRIDE = 16;
 constexpr int EST_PARTS = 8;      // most blocks that share a walker's estimators
 
+inline int sm_count() {
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+
 // f(w0, n) for spans [w0, w0 + n) of the walkers: launches with the walkers along y or z of
 // the grid, which end at 65,535.
 template <typename F>

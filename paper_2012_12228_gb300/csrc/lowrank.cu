@@ -375,8 +375,11 @@ __global__ void __launch_bounds__(LR_THREADS) k_green_lr(const double2* __restri
     }
 }
 
-int lr_threads(int M) {
-    int t = 2 * (((M + 31) / 32) * 32);          // two lanes per column of a reflector's update
+// Two lanes per column of a reflector's update while an SM has two walkers at most; with more,
+// smaller blocks let more of them run at once (G and QRCP of ten slices: M = 81, 608 walkers 42.9
+// and 15.2 ms with two lanes, 29.9 and 15.3 with one; M = 33, 2432 walkers 59.6 and 6.5, 51.0 and 6.1).
+int lr_threads(int M, int W) {
+    int t = (W <= 2 * sm_count() ? 2 : 1) * (((M + 31) / 32) * 32);
     return t > LR_THREADS ? LR_THREADS : (t < 32 ? 32 : t);
 }
 
@@ -387,7 +390,7 @@ cudaError_t launch_qrcp_lr(ftq_ctx* c) {
     const size_t sm = (sizeof(double) + sizeof(int)) * M;
     {
         LaunchScope ls(c, FTQ_K_QRCP);
-        k_qrcp_lr<<<c->W, lr_threads(M), sm, c->stream>>>(c->Y, c->zbuf[0], c->work, c->work2, c->DR, c->Tinv, c->hh,
+        k_qrcp_lr<<<c->W, lr_threads(M, c->W), sm, c->stream>>>(c->Y, c->zbuf[0], c->work, c->work2, c->DR, c->Tinv, c->hh,
                                                          c->htau, c->wstate, c->status, M, c->opts.low_rank_threshold);
     }
     double2* qn = c->zbuf[0];
@@ -407,7 +410,7 @@ cudaError_t launch_green_lr(ftq_ctx* c, const double2* Y, int k, bool update, bo
     }
     const double lscale = physical ? 0.0 : left_scale(c, k);
     LaunchScope ls(c, FTQ_K_GREEN);
-    k_green_lr<<<c->W, lr_threads(M), sm, c->stream>>>(Y, c->Tinv, c->DR, c->work, c->work2, c->zbuf[0], c->zbuf[1],
+    k_green_lr<<<c->W, lr_threads(M, c->W), sm, c->stream>>>(Y, c->Tinv, c->DR, c->work, c->work2, c->zbuf[0], c->zbuf[1],
                                                       c->G, c->hh, c->htau, c->tab.eps, c->wstate, c->status, M,
                                                       lscale, c->sys.mu_T, c->opts.low_rank_threshold,
                                                       c->opts.constraint, update ? 1 : 0, physical ? 0 : 1,
