@@ -105,12 +105,13 @@ __global__ void __launch_bounds__(1024) k_est_walkers(const T* __restrict__ G, c
         }
         for (int q = part + (int)threadIdx.x * nparts; q < nqh; q += blockDim.x * nparts)
             e2 = e2 + cmul(rho[1 + 2 * q], rho[2 + 2 * q]) * (4.0 * vq[q]);
-        // The units shorten along the list: every other round of the warps of all parts runs
-        // backwards, so that each warp, and with it each part, gets about the same work (complex128,
-        // M = 171, one block per walker: 2.13 -> 1.38 ms).
+        // The units shorten along the list: with complex128 G every other round of the warps of all
+        // parts runs backwards, so that each warp, and with it each part, gets about the same work
+        // (M = 171, one block per walker: 2.13 -> 1.38 ms).  FP32 G goes forwards only: the caches
+        // bound it, not the longest warp (M = 257, 1024 walkers 8.36 ms, 8.62 with turns).
         const int round = nw * nparts, t = warp * nparts + part;
         for (int u0 = 0, back = 0; u0 < nunits; u0 += round, back ^= 1) {
-            const int u = u0 + (back ? round - 1 - t : t);
+            const int u = u0 + (sizeof(T) == sizeof(double2) && back ? round - 1 - t : t);
             if (u >= nunits) continue;
             const int4 un = units[u];                  // slot pairs [x, y), chunk from z, v_Q index w
             const int f = un.z + lane;
